@@ -1,8 +1,6 @@
 // ExtractSG state shared by the pipeline stages.
 #pragma once
 
-#include <vector>
-
 #include "graph.cuh"
 
 namespace lds {
@@ -11,10 +9,12 @@ struct SgState {
     int64_t D = 0;                        // denominator of the loads
     DevBuf<int32_t> order;                // [n] internal ids by (load desc, id asc)
     DevBuf<int32_t> pos;                  // [n] position of each internal id
-    std::vector<int64_t> cuts;            // 1-based cut positions (ascending)
-    std::vector<int64_t> group_end;       // exclusive end position of each accepted group
-    std::vector<long long> lo, hi;        // min / max modified load of each group (over D)
-    int64_t chain_checks = 0;             // single checks of merged candidates
+    int64_t ncut = 0;
+    DevBuf<int64_t> cuts;                 // [ncut] 1-based cut positions (ascending)
+    int32_t ng = 0;                       // accepted groups
+    DevBuf<int64_t> gend;                 // [ng] exclusive end position of each accepted group
+    DevBuf<int64_t> lo, hi;               // [ng] min / max modified load of each group (over D)
+    int32_t windows = 0, steps = 0;       // of the candidate walk
 };
 
 // Alg. 2 on the last Frank-Wolfe run of g (g->fw_*).

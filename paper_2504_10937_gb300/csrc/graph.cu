@@ -120,43 +120,8 @@ __global__ void copy_unflagged_kernel(const int32_t* col, int32_t* fwcol, int64_
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < k2; s += stride) fwcol[s] = col[s];
 }
 
-// upper slot of edge e = (u, v), u < v: row u lists its lower neighbours first, then
-// its upper ones in edge order, so the slot is rowptr[u] + low(u) + (e - eptr[u])
-__global__ void slot_edge_upper_kernel(const int32_t* eu, int64_t m, const int64_t* rowptr, const int64_t* updeg,
-                                       const int64_t* eptr, int64_t* slot_edge) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-        const int32_t u = eu[e];
-        const int64_t low = rowptr[u + 1] - rowptr[u] - updeg[u];
-        slot_edge[rowptr[u] + low + (e - eptr[u])] = e;
-    }
-}
-
-__global__ void second_endpoint_keys_kernel(const int32_t* ev, int64_t m, uint64_t* key, uint32_t* eid) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-        key[e] = (uint64_t)ev[e];
-        eid[e] = (uint32_t)e;
-    }
-}
-
-// lower slots: the edges sorted (stably) by their upper endpoint v, so by u within v;
-// the i-th of v's group sits at slot rowptr[v] + (i - gstart[v])
-__global__ void slot_edge_lower_kernel(const uint64_t* key, const uint32_t* eid, int64_t m, const int64_t* rowptr,
-                                       const int64_t* gstart, int64_t* slot_edge) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) {
-        const int64_t v = (int64_t)key[i];
-        slot_edge[rowptr[v] + (i - gstart[v])] = (int64_t)eid[i];
-    }
-}
-
-__global__ void lower_degree_kernel(const int64_t* rowptr, const int64_t* updeg, int32_t nact, int64_t* low) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nact; r += stride)
-        low[r] = rowptr[r + 1] - rowptr[r] - updeg[r];
-}
-
+// upper neighbours of every row; the row lists its lower neighbours first, then its
+// upper ones in canonical edge order
 __global__ void upper_degree_kernel(const int64_t* rowptr, const int32_t* col, int32_t nact, int64_t* updeg) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nact; r += stride) {
@@ -167,6 +132,14 @@ __global__ void upper_degree_kernel(const int64_t* rowptr, const int32_t* col, i
         }
         updeg[r] = e - lo;
     }
+}
+
+// the first upper slot of row x, rowptr[x + 1] - updeg[x], is canonical edge eptr[x]
+__global__ void edge_shift_kernel(const int64_t* rowptr, const int64_t* updeg, const int64_t* eptr, int32_t nact,
+                                  int64_t* shift) {
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride)
+        shift[x] = eptr[x] - (rowptr[x + 1] - updeg[x]);
 }
 
 __global__ void map_ids_kernel(const int32_t* in, const int32_t* map, int64_t k, int32_t* out) {
@@ -188,26 +161,15 @@ void map_ids(const int32_t* in, const int32_t* map, int64_t k, int32_t* out, cud
     LDS_CHECK_LAUNCH();
 }
 
-void ensure_slot_edge(lds_graph* g) {
-    if (g->slot_edge.p || g->m == 0) return;
+void ensure_edge_shift(lds_graph* g) {
+    if (g->edge_shift.p || g->m == 0) return;
     cudaStream_t s = g->stream;
     DevBuf<int64_t> updeg(g->nact, s), eptr(g->nact, s);
     LDS_LAUNCH(upper_degree_kernel, grid_for(g->nact, 256), 256, 0, s, g->rowptr.get(), g->col.get(), g->nact, updeg.get());
-    LDS_CHECK_LAUNCH();
     exclusive_scan_i64_dev(updeg.get(), eptr.get(), g->nact, nullptr, s);
-    g->slot_edge.alloc(2 * g->m, s);
-    const int64_t m = g->m;
-    LDS_LAUNCH(slot_edge_upper_kernel, grid_for(m, 256), 256, 0, s, g->eu.get(), m, g->rowptr.get(), updeg.get(),
-               eptr.get(), g->slot_edge.get());
-    DevBuf<int64_t> low(g->nact, s), gstart(g->nact, s);
-    LDS_LAUNCH(lower_degree_kernel, grid_for(g->nact, 256), 256, 0, s, g->rowptr.get(), updeg.get(), g->nact, low.get());
-    exclusive_scan_i64_dev(low.get(), gstart.get(), g->nact, nullptr, s);
-    DevBuf<uint64_t> key(m, s);
-    DevBuf<uint32_t> eid(m, s);
-    LDS_LAUNCH(second_endpoint_keys_kernel, grid_for(m, 256), 256, 0, s, g->ev.get(), m, key.get(), eid.get());
-    radix_sort_u64(key.get(), eid.get(), m, std::max(1, bit_length_u64((uint64_t)g->nact)), s);
-    LDS_LAUNCH(slot_edge_lower_kernel, grid_for(m, 256), 256, 0, s, key.get(), eid.get(), m, g->rowptr.get(),
-               gstart.get(), g->slot_edge.get());
+    g->edge_shift.alloc(g->nact, s);
+    LDS_LAUNCH(edge_shift_kernel, grid_for(g->nact, 256), 256, 0, s, g->rowptr.get(), updeg.get(), eptr.get(), g->nact,
+               g->edge_shift.get());
 }
 
 void to_original_order_i64(const lds_graph* g, const int64_t* in_int, int64_t* out_orig) {
@@ -369,7 +331,7 @@ void set_stream(lds_graph* g, cudaStream_t s) {
     g->col.s = s;
     g->fwcol.s = s;
     g->chunk_row0.s = s;
-    g->slot_edge.s = s;
+    g->edge_shift.s = s;
     g->ta.s = s;
     g->tb.s = s;
     g->tc.s = s;

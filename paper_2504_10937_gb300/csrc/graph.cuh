@@ -23,7 +23,8 @@ struct lds_graph {
     lds::DevBuf<int32_t> col;         // [2m] internal ids, ascending in each row
     lds::DevBuf<int32_t> fwcol;       // [2m] col with bit 31 set on the first slot of each row
     lds::DevBuf<int32_t> chunk_row0;  // [ceil(2m / 32)] row of slot 32 g
-    lds::DevBuf<int64_t> slot_edge;   // [2m] canonical edge id of each slot (lazy)
+    // [nact] (lazy): slot q of row x with col[q] > x is canonical edge q + edge_shift[x]
+    lds::DevBuf<int64_t> edge_shift;
 
     // triangles (lazy): internal ids a < b < c, triangle order
     int64_t ntri = -1;
@@ -76,8 +77,8 @@ namespace lds {
 // work on the previous stream is pending.
 void set_stream(lds_graph* g, cudaStream_t s);
 
-// Builds slot_edge (canonical edge id of every CSR slot) if not present.
-void ensure_slot_edge(lds_graph* g);
+// Builds edge_shift if not present.
+void ensure_edge_shift(lds_graph* g);
 
 // Runs `iters` Frank-Wolfe iterations and leaves the results in g->fw_*.
 void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool want_last);

@@ -395,24 +395,17 @@ struct Driver {
         SgState sg;
         extract_sg(h, sg);
         const int32_t n = h->n;
-        const int32_t ng = (int32_t)sg.group_end.size();
-        DevBuf<int64_t> gend(std::max(ng, 1), s), lo(std::max(ng, 1), s), hi(std::max(ng, 1), s);
-        if (ng) {
-            std::vector<int64_t> l(sg.lo.begin(), sg.lo.end()), hh(sg.hi.begin(), sg.hi.end());
-            copy_in(gend.get(), sg.group_end.data(), LDS_MEM_HOST, ng * sizeof(int64_t), s);
-            copy_in(lo.get(), l.data(), LDS_MEM_HOST, ng * sizeof(int64_t), s);
-            copy_in(hi.get(), hh.data(), LDS_MEM_HOST, ng * sizeof(int64_t), s);
-            int64_t npos = sg.group_end.back();
-            LDS_LAUNCH(apply_groups_kernel, grid_for(npos, DB), DB, 0, s, sg.order.get(), gend.get(), lo.get(), hi.get(),
-                       ng, sg.D, npos, b.un.get(), b.ud.get(), b.ln.get(), b.ld.get());
-        }
+        const int32_t ng = sg.ng;
+        if (ng)
+            LDS_LAUNCH(apply_groups_kernel, grid_for(n, DB), DB, 0, s, sg.order.get(), sg.gend.get(), sg.lo.get(),
+                       sg.hi.get(), ng, sg.D, n, b.un.get(), b.ud.get(), b.ln.get(), b.ld.get());
         auto t2 = std::chrono::steady_clock::now();
         DevBuf<uint8_t> status(std::max(n, 1), s);
         prune(h, tri, b.un.get(), b.ud.get(), b.ln.get(), b.ld.get(), status.get());
         // kept members per group (the remainder is one more group)
         DevBuf<int32_t> gid(std::max(n, 1), s), keep(std::max(n, 1), s), gcount(ng + 1, s);
         LDS_CUDA(cudaMemsetAsync(gcount.get(), 0, (ng + 1) * sizeof(int32_t), s));
-        if (n) LDS_LAUNCH(group_keys_kernel, grid_for(n, DB), DB, 0, s, sg.order.get(), gend.get(), ng, n, status.get(),
+        if (n) LDS_LAUNCH(group_keys_kernel, grid_for(n, DB), DB, 0, s, sg.order.get(), sg.gend.get(), ng, n, status.get(),
                           gid.get(), keep.get(), gcount.get());
         DevBuf<int64_t> kpos(std::max(n, 1), s);
         int64_t nk = exclusive_scan_i32_to_i64(keep.get(), kpos.get(), n, s);

@@ -128,6 +128,10 @@ int64_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cu
     return h;
 }
 
+void exclusive_scan_i32_dev(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s) {
+    scan_impl<int32_t>(in, out, n, nullptr, s);
+}
+
 // ------------------------------------------------------------------ radix sort
 
 namespace {

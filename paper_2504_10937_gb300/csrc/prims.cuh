@@ -16,6 +16,9 @@ void exclusive_scan_i64_dev(const int64_t* in, int64_t* out, int64_t n, int64_t*
 // int32 input flags / counts, int64 exclusive sums.
 int64_t exclusive_scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s);
 
+// int32 input, int64 exclusive sums, no host read-back.
+void exclusive_scan_i32_dev(const int32_t* in, int64_t* out, int64_t n, cudaStream_t s);
+
 // Stable LSD radix sort of uint64 keys on bits [0, bits), 8 bits per pass,
 // with an optional uint32 payload.  keys / vals are sorted in place (a
 // temporary ping-pong buffer is allocated).  vals may be null.

@@ -86,7 +86,7 @@ __global__ void edge_pat_count_kernel(const int32_t* list, int32_t k, int32_t na
 // lower endpoint x and D - W for y
 __global__ void edge_pat_fill_kernel(const int32_t* list, int32_t k, int32_t nact, const int64_t* rowptr,
                                      const int32_t* col, const uint8_t* in, const int32_t* local, const int64_t* off,
-                                     int32_t* pidx, const int64_t* slot_edge, const int64_t* W, int64_t D,
+                                     int32_t* pidx, const int64_t* edge_shift, const int64_t* W, int64_t D,
                                      int64_t* share) {
     WARP_MEMBER_LOOP(k) {
         const int32_t x = list[i];
@@ -107,7 +107,7 @@ __global__ void edge_pat_fill_kernel(const int32_t* list, int32_t k, int32_t nac
                 pidx[2 * at] = (int32_t)i;
                 pidx[2 * at + 1] = local[y];
                 if (share) {
-                    const int64_t w = W[slot_edge[q]];
+                    const int64_t w = W[q + edge_shift[x]];
                     share[2 * at] = w;
                     share[2 * at + 1] = D - w;
                 }
@@ -493,7 +493,7 @@ static int64_t build_patterns(lds_graph* g, bool tri, const int32_t* list, int32
         pptr.alloc(np + 1, s);
         pidx.alloc(std::max<int64_t>(2 * ne + nl, 1), s);
         if (warm) {
-            ensure_slot_edge(g);
+            ensure_edge_shift(g);
             share->alloc(std::max<int64_t>(2 * ne + nl, 1), s);
         }
         int64_t* sh = warm ? share->get() : nullptr;
@@ -507,7 +507,7 @@ static int64_t build_patterns(lds_graph* g, bool tri, const int32_t* list, int32
         }
         if (k && ne)
             LDS_LAUNCH(edge_pat_fill_kernel, grid_for((int64_t)k * 32, VB), VB, 0, s, list, k, nact, g->rowptr.get(), g->col.get(),
-                       sc.in.get(), sc.local.get(), off.get(), pidx.get(), warm ? g->slot_edge.get() : nullptr,
+                       sc.in.get(), sc.local.get(), off.get(), pidx.get(), warm ? g->edge_shift.get() : nullptr,
                        warm ? g->fw_W.get() : nullptr, g->fw_D, sh);
         if (k && nl)
             LDS_LAUNCH(loop_fill_kernel, grid_for(k, VB), VB, 0, s, lcnt.get(), loff.get(), k, pidx.get(), 2 * ne, sh);

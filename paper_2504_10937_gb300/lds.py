@@ -177,7 +177,7 @@ def set_flow_variant(variant: int):
 
 
 def set_extract_variant(variant: int):
-    """0: automatic; 1: the large-graph ExtractSG walk (device chains) at every size."""
+    """0: windows of up to 32 candidates; 1: windows of one candidate."""
     _check(load().lds_set_extract_variant(int(variant)))
 
 
