@@ -134,6 +134,8 @@ __global__ void tri_rows_orig_kernel(const int32_t* ta, const int32_t* tb, const
 
 // ---- peeling
 
+constexpr int32_t PEEL_DEAD = -(1 << 30);   // count of a vertex that is peeled or outside the mask
+
 __global__ void alive_init_kernel(const uint8_t* init, int32_t nact, uint8_t* alive, int64_t* core, int32_t* nalive) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int32_t c = 0;
@@ -146,15 +148,29 @@ __global__ void alive_init_kernel(const uint8_t* init, int32_t nact, uint8_t* al
     if (c) atomicAdd(nalive, c);
 }
 
+// one warp per vertex: live neighbours
 __global__ void alive_degree_kernel(const int64_t* rowptr, const int32_t* col, const uint8_t* alive, int32_t nact,
                                     int32_t* deg) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride) {
-        if (!alive[x]) continue;
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < nact; x += nwarps) {
+        if (!alive[x]) {
+            // stays negative when every neighbour takes one off it
+            if (lane == 0) deg[x] = INT_MIN + (int32_t)(rowptr[x + 1] - rowptr[x]);
+            continue;
+        }
         int32_t d = 0;
-        for (int64_t q = rowptr[x], e = rowptr[x + 1]; q < e; ++q) d += alive[col[q]];
-        deg[x] = d;
+        for (int64_t q = rowptr[x] + lane, e = rowptr[x + 1]; q < e; q += 32) d += alive[col[q]];
+        d = __reduce_add_sync(0xffffffffu, d);
+        if (lane == 0) deg[x] = d;
     }
+}
+
+// every listed pattern of a live vertex is live: its count is its list's length
+__global__ void full_count_kernel(const int64_t* ptr, const uint8_t* alive, int32_t nact, int32_t* deg) {
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride)
+        deg[x] = alive[x] ? (int32_t)(ptr[x + 1] - ptr[x]) : PEEL_DEAD;
 }
 
 // triangle counts of G[alive]; triangles with a dead vertex are marked dead
@@ -201,385 +217,489 @@ __device__ __forceinline__ unsigned long long agg_slot(unsigned long long* ctr) 
     return grp.shfl(base, 0) + grp.thread_rank();
 }
 
-// Removing a peeled vertex at level k lowers the count of each neighbour (of
-// each other vertex of each live triangle); a vertex whose count falls from
-// k + 1 to k is peeled at level k too (exactly one decrement sees k + 1) and
-// joins the next frontier.  Counts of vertices already peeled are lowered as
-// well: theirs are at most their level <= k and only fall, so they never see
-// k + 1 again, and skipping a liveness test saves a dependent load.
-__device__ __forceinline__ void peel_drop(int32_t y, int64_t k, uint8_t* alive, int32_t* deg, int64_t* core,
-                                          int32_t* next, unsigned long long* next_cnt) {
-    if ((int64_t)atomicSub(deg + y, 1) == k + 1) {
-        alive[y] = 0;
-        core[y] = k;
-        next[agg_slot(next_cnt)] = y;
+__global__ void mark_dead_kernel(const uint8_t* alive, int32_t nact, int32_t* deg) {
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride)
+        if (!alive[x]) deg[x] = PEEL_DEAD;
+}
+
+// A frontier is a queue of chunks: up to PEEL_CHUNK incidences of one peeled
+// vertex, taken by one warp, so a hub is shared by the whole grid.
+constexpr int PEEL_CHUNK = 64;
+struct __align__(16) PeelChunk {
+    int64_t start;
+    int32_t len, x;
+};
+
+// The lanes with `want` append the chunks of their vertex y (whole warp calls).
+__device__ __forceinline__ void peel_push(bool want, int32_t y, const int64_t* ptr, PeelChunk* Q,
+                                          unsigned long long* cnt, int lane) {
+    unsigned mask = __ballot_sync(0xffffffffu, want);
+    if (!mask) return;
+    int64_t b = 0;
+    int32_t len = 0;
+    if (want) {
+        b = ptr[y];
+        len = (int32_t)(ptr[y + 1] - b);
+    }
+    const int32_t nch = (len + PEEL_CHUNK - 1) / PEEL_CHUNK;
+    int32_t incl = nch;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    unsigned long long base = 0;
+    if (lane == 31 && incl) base = atomicAdd(cnt, (unsigned long long)incl);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    for (; mask; mask &= mask - 1) {
+        const int l = __ffs(mask) - 1;
+        const int32_t vy = __shfl_sync(0xffffffffu, y, l), vlen = __shfl_sync(0xffffffffu, len, l);
+        const int64_t vb = __shfl_sync(0xffffffffu, b, l);
+        const int32_t vn = __shfl_sync(0xffffffffu, nch, l), ve = __shfl_sync(0xffffffffu, incl, l);
+        for (int32_t c = lane; c < vn; c += 32) {
+            PeelChunk e{vb + (int64_t)c * PEEL_CHUNK, min(PEEL_CHUNK, vlen - c * PEEL_CHUNK), vy};
+            Q[base + (unsigned long long)(ve - vn + c)] = e;
+        }
     }
 }
-
-__device__ __forceinline__ void peel_triangle(int32_t t, int32_t x, int64_t k, const int32_t* ta, const int32_t* tb,
-                                              const int32_t* tc, uint8_t* tdead, uint8_t* alive, int32_t* deg,
-                                              int64_t* core, int32_t* next, unsigned long long* next_cnt) {
-    unsigned int* word = (unsigned int*)(tdead + (t & ~3));
-    unsigned int bit = 1u << (8 * (t & 3));
-    if (atomicOr(word, bit) & bit) return;          // the triangle died with another vertex
-    int32_t a = ta[t], b = tb[t], c = tc[t];
-    if (a != x) peel_drop(a, k, alive, deg, core, next, next_cnt);
-    if (b != x) peel_drop(b, k, alive, deg, core, next, next_cnt);
-    if (c != x) peel_drop(c, k, alive, deg, core, next, next_cnt);
-}
-
-constexpr int PEEL_LIGHT = 8;       // a lane removes a vertex with at most this many incidences
-constexpr int PEEL_CHUNK = 128;     // otherwise a warp removes each chunk of this many (4 per lane)
 
 constexpr int PEEL_SOLO = 8192;      // live vertices the one-block kernel finishes with, in shared memory
 constexpr int PEEL_SOLO_T = 1024;    // its threads
-constexpr size_t PEEL_SOLO_SMEM = 16 + (size_t)PEEL_SOLO * (4 * sizeof(int32_t) + 1);
+constexpr int SOLO_CHUNK = 128;      // neighbours a warp takes at a time (4 per lane)
+constexpr size_t PEEL_SOLO_SMEM = (size_t)PEEL_SOLO * (4 + 4 + 2 * 2 + 2 * 4) + 16;
 
-// exclusive block scan of one int64 per thread (PEEL_SOLO_T threads); returns the total
-__device__ __forceinline__ int64_t block_scan_i64(int64_t v, int64_t* out, int64_t* wsum) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    int64_t inc = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) wsum[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        int64_t w = wsum[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t t = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += t;
-        }
-        wsum[lane] = w;                          // inclusive warp totals
-    }
-    __syncthreads();
-    out[tid] = inc - v + (wid ? wsum[wid - 1] : 0);
-    const int64_t total = wsum[31];
-    __syncthreads();
-    return total;
-}
+// ctrl words of a peel
+constexpr int PC_Q = 0;        // [3] chunk counts of the queues
+constexpr int PC_ERR = 3;      // step bound hit
+constexpr int PC_LIST = 4;     // [3] live-list counts
+constexpr int PC_MIN = 7;      // [3] lower bound of the live counts
+constexpr int PC_STEPS = 10;   // steps and last level (reported)
+constexpr int PC_LEVEL = 11;
+constexpr int PC_SOLO = 12;    // hand-over: flag, list, live count, level, steps
+constexpr int PC_WORDS = 17;
 
-// The dense tail of the peel, in one block, once at most PEEL_SOLO vertices are
-// live (the grid-wide kernel hands over through ctrl[9..12]).  Their counts, live
-// flags and the frontiers sit in shared memory (live vertex x at slot[x]; slot
-// is -1 for every other vertex, whose count no longer matters), so a round costs
-// block barriers and shared-memory atomics instead of grid barriers and L2
-// atomics.  A round's incidences are spread evenly over the threads (batches of
-// PEEL_SOLO_T frontier vertices, a scan of their incidence counts), so one hub
-// does not hold the round.  Same levels and rules as the grid-wide loop.
+// A peel in one block: the dense tail of an edge peel once at most PEEL_SOLO
+// vertices are live (SOLO_TAIL, handed over by the grid-wide kernel), or a whole
+// small graph (SOLO_EDGES, SOLO_TRIS).  For the tail the live subgraph was
+// compacted to 16-bit local ids (cadj, rows at coff, padded to whole 4-entry
+// groups with 0xffff), so a round reads live neighbours only; a whole graph's rows
+// are used as they are, vertex x being slot x.  Counts, frontiers and the dead
+// bits of triangles sit in shared memory.  A frontier entry is a vertex and the
+// number of 128-incidence chunks before it, both handed out by one 64-bit shared
+// atomic; warps find their chunk's vertex by a 32-way search.  One block barrier
+// per round.  Same levels and rules as the grid-wide kernel.
+//
+// Bounded by the chain of one round (row entry from L2, shared count, frontier) in
+// one SM: 1.0-1.5 us a step where grid barriers make it 4 or more.  The one-block
+// tail over uncompacted rows took 8.7 us a step on the 1M-vertex power-law graph.
+enum SoloKind { SOLO_TAIL, SOLO_EDGES, SOLO_TRIS };
+constexpr int64_t PEEL_SOLO_TRIS = 1 << 19;     // most triangles of SOLO_TRIS (their dead bits: 64 KB)
+constexpr size_t PEEL_SOLO_TRIS_SMEM = PEEL_SOLO_SMEM + PEEL_SOLO_TRIS / 8;
+
+template <SoloKind KIND>
 __global__ void __launch_bounds__(PEEL_SOLO_T, 1) peel_solo_kernel(
-    bool tri, const int64_t* ptr, const int32_t* adj, const int32_t* ta, const int32_t* tb, const int32_t* tc,
-    uint8_t* tdead, const uint8_t* alive, const int32_t* deg, int64_t* core, const int32_t* A0, const int32_t* A1,
-    int32_t* slot, unsigned long long* ctrl, int64_t max_steps) {
+    const int32_t* A0, const int32_t* A1, const int32_t* deg, const int32_t* coff, const uint16_t* cadj, int32_t n,
+    const int64_t* ptr, const int32_t* __restrict__ adj, const int32_t* __restrict__ ta,
+    const int32_t* __restrict__ tb, const int32_t* __restrict__ tc, const uint8_t* __restrict__ tdead, int64_t nt,
+    int64_t* core, unsigned long long* ctrl, int64_t max_steps) {
     extern __shared__ __align__(16) unsigned char psm[];
-    __shared__ int64_t b_off[PEEL_SOLO_T], b_beg[PEEL_SOLO_T], wsum[32];
-    __shared__ int32_t b_x[PEEL_SOLO_T];
-    if (ctrl[12] == 0) return;                  // the grid-wide kernel finished the peel
-    const int32_t* list = ctrl[9] ? A1 : A0;
-    const int32_t nl = (int32_t)ctrl[4 + ctrl[9]];
-    int64_t k = (int64_t)ctrl[10], steps = (int64_t)ctrl[11];
-    int32_t* sc = reinterpret_cast<int32_t*>(psm);              // [0] frontier count, [1] smallest kept count
-    int32_t* sv = sc + 4;                                         // vertex of each slot
-    int32_t* sd = sv + PEEL_SOLO;                                 // its count
-    int32_t* fa = sd + PEEL_SOLO;                                 // frontiers (slots)
-    int32_t* fb = fa + PEEL_SOLO;
-    uint8_t* sl = reinterpret_cast<uint8_t*>(fb + PEEL_SOLO);     // live flag
-    const int tid = threadIdx.x, bd = blockDim.x;
+    __shared__ unsigned long long q[3];
+    __shared__ int32_t smin[3];
+    if (KIND == SOLO_TAIL && ctrl[PC_SOLO] == 0) return;   // the grid-wide kernel finished the peel
+    const int32_t* list = KIND == SOLO_TAIL ? (ctrl[PC_SOLO + 1] ? A1 : A0) : nullptr;
+    const int32_t nl = KIND == SOLO_TAIL ? (int32_t)ctrl[PC_SOLO + 2] : n;
+    int32_t k = KIND == SOLO_TAIL ? (int32_t)ctrl[PC_SOLO + 3] : 0;
+    int64_t steps = KIND == SOLO_TAIL ? (int64_t)ctrl[PC_SOLO + 4] : 0;
+    int32_t* sd = reinterpret_cast<int32_t*>(psm);                // live count (negative once peeled)
+    int32_t* off = sd + PEEL_SOLO;                                // [nl + 1] row starts
+    int32_t* fo = off + PEEL_SOLO + 4;                            // [2][PEEL_SOLO] chunks before a frontier entry
+    uint16_t* fv = reinterpret_cast<uint16_t*>(fo + 2 * PEEL_SOLO);   // [2][PEEL_SOLO] its vertex
+    uint32_t* dead = reinterpret_cast<uint32_t*>(fv + 2 * PEEL_SOLO); // SOLO_TRIS: one bit per triangle
+    const int tid = threadIdx.x, bd = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = bd >> 5;
     for (int i = tid; i < nl; i += bd) {
-        const int32_t x = list[i];
-        sv[i] = x;
-        sd[i] = deg[x];
-        sl[i] = alive[x];
-        slot[x] = i;
+        const int32_t d = deg[KIND == SOLO_TAIL ? list[i] : i];
+        sd[i] = KIND == SOLO_TAIL && d < 0 ? PEEL_DEAD : d;
+    }
+    for (int i = tid; i <= nl; i += bd) off[i] = KIND == SOLO_TAIL ? coff[i] : (int32_t)ptr[i];
+    if (KIND == SOLO_TRIS)
+        // triangles with a vertex outside the mask are dead from the start
+        for (int64_t t = tid; t < ((nt + 31) & ~31ll); t += bd) {
+            const unsigned m = __ballot_sync(0xffffffffu, t < nt && tdead[t]);
+            if (lane == 0) dead[t >> 5] = m;
+        }
+    if (tid < 3) {
+        q[tid] = 0;
+        smin[tid] = INT_MAX;
     }
     __syncthreads();
+    int ph = 0, lv = 0;                          // queue phase and level, modulo 3 for the counters
+    // vertex i is peeled at level k: core number, and its row joins the next frontier
+    auto peel = [&](int i) {
+        core[KIND == SOLO_TAIL ? list[i] : i] = k;
+        const unsigned nch = (unsigned)(off[i + 1] - off[i] + SOLO_CHUNK - 1) / SOLO_CHUNK;
+        if (nch == 0) return;
+        const unsigned long long o = atomicAdd(&q[(ph + 1) % 3], ((unsigned long long)nch << 32) | 1ull);
+        const int at = ((ph + 1) & 1) * PEEL_SOLO + (int)(unsigned)o;
+        fv[at] = (uint16_t)i;
+        fo[at] = (int32_t)(o >> 32);
+    };
+    int32_t mn = INT_MAX;
+    // a vertex whose count falls from k + 1 to k is peeled at k
+    auto drop = [&](int y) {
+        const int32_t old = atomicSub(sd + y, 1);
+        if (old == k + 1) {
+            sd[y] = PEEL_DEAD;
+            peel(y);
+        } else if (old > k) {
+            mn = min(mn, old - 1);
+        }
+    };
     for (;;) {
         if (++steps > max_steps) {
-            if (tid == 0) ctrl[3] = 1;
+            if (tid == 0) ctrl[PC_ERR] = 1;
             return;
         }
         if (tid == 0) {
-            sc[0] = 0;
-            sc[1] = INT_MAX;
+            q[(ph + 2) % 3] = 0;
+            smin[(lv + 1) % 3] = INT_MAX;
         }
-        __syncthreads();
-        // level scan: live vertices with count <= k are peeled at k
-        for (int i = tid; i < nl; i += bd)
-            if (sl[i]) {
-                const int32_t d = sd[i];
-                if (d <= k) {
-                    sl[i] = 0;
-                    core[sv[i]] = k;
-                    fa[atomicAdd(sc, 1)] = i;
-                } else {
-                    atomicMin(sc + 1, d);
-                }
+        // level scan
+        bool kept = false;
+        mn = INT_MAX;
+        for (int i = tid; i < nl; i += bd) {
+            const int32_t d = sd[i];
+            if (d < 0) continue;
+            if (d <= k) {
+                sd[i] = PEEL_DEAD;
+                peel(i);
+            } else {
+                kept = true;
+                mn = min(mn, d);
             }
-        __syncthreads();
-        int32_t nf = sc[0];
-        const int32_t mn = sc[1];
-        __syncthreads();
-        if (nf == 0) {
-            if (mn == INT_MAX) {
-                if (tid == 0) {
-                    ctrl[6] = (unsigned long long)steps;
-                    ctrl[7] = (unsigned long long)k;
-                }
-                return;
-            }
-            k = max(k + 1, (int64_t)mn);
-            continue;
         }
-        int32_t* cf = fa;
-        int32_t* nx = fb;
-        while (nf > 0) {
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        if (lane == 0 && mn != INT_MAX) atomicMin(&smin[lv % 3], mn);
+        const bool more = __syncthreads_or(kept) != 0;
+        ++ph;
+        unsigned long long cur = q[ph % 3];
+        while (cur) {
             if (++steps > max_steps) {
-                if (tid == 0) ctrl[3] = 1;
+                if (tid == 0) ctrl[PC_ERR] = 1;
                 return;
             }
-            if (tid == 0) sc[0] = 0;
-            __syncthreads();
-            // a vertex whose count falls from k + 1 to k is peeled at k
-            auto drop = [&](int32_t y) {
-                const int32_t j = slot[y];
-                if (j >= 0 && atomicSub(sd + j, 1) == k + 1) {
-                    sl[j] = 0;
-                    core[y] = k;
-                    nx[atomicAdd(sc, 1)] = j;
+            if (tid == 0) q[(ph + 2) % 3] = 0;
+            const int nf = (int)(unsigned)cur, nc = (int)(cur >> 32);
+            const int32_t* cfo = fo + (ph & 1) * PEEL_SOLO;
+            const uint16_t* cfv = fv + (ph & 1) * PEEL_SOLO;
+            mn = INT_MAX;
+            for (int c = wid; c < nc; c += nw) {
+                int lo = 0, cnt = nf;                  // last entry with fo <= c
+                while (cnt > 1) {
+                    const int st = (cnt + 31) >> 5, at = lane * st;
+                    const unsigned m = __ballot_sync(0xffffffffu, at < cnt && cfo[lo + at] <= c);
+                    const int j = 31 - __clz(m);
+                    lo += j * st;
+                    cnt = min(st, cnt - j * st);
                 }
-            };
-            for (int32_t base = 0; base < nf; base += bd) {
-                const int32_t j = base + tid;
-                int64_t d = 0, b0 = 0;
-                int32_t x = -1;
-                if (j < nf) {
-                    x = sv[cf[j]];
-                    b0 = ptr[x];
-                    d = ptr[x + 1] - b0;
-                }
-                const int64_t total = block_scan_i64(d, b_off, wsum);
-                b_x[tid] = x;
-                b_beg[tid] = b0;
-                __syncthreads();
-                const int32_t cnt = min(bd, nf - base);
-                for (int64_t i = tid; i < total; i += bd) {
-                    int32_t lo = 0, hi = cnt;            // last entry with offset <= i
-                    while (hi - lo > 1) {
-                        const int32_t mid = (lo + hi) >> 1;
-                        if (b_off[mid] <= i) lo = mid; else hi = mid;
+                const int i = cfv[lo];
+                const int32_t e = off[i + 1], b = off[i] + (c - cfo[lo]) * SOLO_CHUNK;
+                if (KIND == SOLO_TAIL) {
+                    if (b + lane * 4 < e) {
+                        const ushort4 v = *reinterpret_cast<const ushort4*>(cadj + b + lane * 4);
+                        const int y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (y[j] != 0xffff) drop(y[j]);
                     }
-                    const int32_t xv = b_x[lo];
-                    const int32_t e = adj[b_beg[lo] + (i - b_off[lo])];
-                    if (!tri) {
-                        drop(e);
+                } else {
+                    int32_t y[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) y[j] = b + 32 * j + lane < e ? adj[b + 32 * j + lane] : -1;
+                    if (KIND == SOLO_EDGES) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (y[j] >= 0) drop(y[j]);
                     } else {
-                        unsigned int* word = (unsigned int*)(tdead + (e & ~3));
-                        const unsigned int bit = 1u << (8 * (e & 3));
-                        if (atomicOr(word, bit) & bit) continue;      // died with another vertex
-                        const int32_t va = ta[e], vb = tb[e], vc = tc[e];
-                        if (va != xv) drop(va);
-                        if (vb != xv) drop(vb);
-                        if (vc != xv) drop(vc);
+                        int32_t v[4][3];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t bit = 1u << (y[j] & 31);
+                            // else it died with another vertex
+                            if (y[j] >= 0 && (atomicOr(dead + (y[j] >> 5), bit) & bit)) y[j] = -1;
+                            if (y[j] >= 0) {
+                                v[j][0] = ta[y[j]];
+                                v[j][1] = tb[y[j]];
+                                v[j][2] = tc[y[j]];
+                            }
+                        }
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (y[j] >= 0) {
+#pragma unroll
+                                for (int r = 0; r < 3; ++r)
+                                    if (v[j][r] != i) drop(v[j][r]);
+                            }
                     }
                 }
-                __syncthreads();
             }
-            nf = sc[0];
+            mn = __reduce_min_sync(0xffffffffu, mn);
+            if (lane == 0 && mn != INT_MAX) atomicMin(&smin[lv % 3], mn);
             __syncthreads();
-            int32_t* t = cf;
-            cf = nx;
-            nx = t;
+            ++ph;
+            cur = q[ph % 3];
         }
-        k = k + 1;
+        if (!more) {
+            if (tid == 0) {
+                ctrl[PC_STEPS] = (unsigned long long)steps;
+                ctrl[PC_LEVEL] = (unsigned long long)k;
+            }
+            return;
+        }
+        k = max(k + 1, smin[lv % 3]);
+        ++lv;
     }
 }
 
 // Whole peeling loop in one cooperative launch (peeling by levels).  A level k
-// starts with a scan of the live-vertex list: vertices with count <= k are
-// peeled (core k) into the frontier, the others go to the other list, and the
-// smallest kept count is recorded; an empty frontier moves k to
-// max(k + 1, that minimum) and scans again.  Frontier rounds then remove the
-// frontier and collect the vertices that fall to k: a lane removes a vertex
-// with few incidences itself, and the incidences of the others are cut into
-// chunks that all warps share, so a hub does not hold up the round.  Once the
-// live list is down to `solo` (at most PEEL_SOLO) vertices, the grid stops and
-// peel_solo_kernel finishes in one block: block barriers cost far less than
-// grid barriers over the many small levels of the dense tail.
-// ctrl: [0..1] frontier counts, [2] smallest kept count, [3] error (bound hit),
-// [4..5] live-list counts, [6..7] steps and last level (reported at the end),
-// [8] chunk count, [9..12] the hand-over (live list, level, steps, flag).  Every
-// thread follows the same k and the same branches: the counters are read right
-// after a barrier.
-__global__ void __launch_bounds__(1024, 1) peel_coop_kernel(bool tri, const int64_t* rowptr, const int32_t* col,
-                                                            const int64_t* vptr, const int32_t* vtri,
-                                                            const int32_t* ta, const int32_t* tb, const int32_t* tc,
-                                                            uint8_t* tdead, uint8_t* alive, int32_t* deg,
-                                                            int64_t* core, int32_t* F0, int32_t* F1, int32_t* A0,
-                                                            int32_t* A1, int32_t* qv, int64_t* qs,
-                                                            unsigned long long* ctrl, int64_t max_steps,
-                                                            int64_t solo) {
+// starts with a scan of the live-vertex list: vertices with count <= k are peeled
+// (core k) and their chunks queued, the others go to the other list.  Rounds then
+// take the queued chunks, one warp each; removing a peeled vertex lowers the count
+// of each neighbour (of each other vertex of each live triangle), and a vertex
+// whose count falls to k is peeled at level k too and queued for the next round.
+// The scan and every drop also keep a lower bound of the live counts, the next
+// level when it is above k + 1.  Peeled vertices hold PEEL_DEAD: their counts stay
+// negative whatever is taken off them.
+//
+// A level of the dense part has little work, so what bounds it is the chain of
+// dependent L2 accesses of a round and its grid barrier.  Every counter is kept
+// three times and used in turn, so one barrier ends a round or a scan, and a queue
+// entry carries its chunk's start and length, so a round is entry -> neighbours ->
+// counts.  (Four barriers a round and a separate pass that queued the chunks of
+// heavy vertices took 16.7 us a step on the R-MAT scale-18 triangles.)
+//
+// An edge peel hands over to peel_solo_kernel once `solo` or fewer vertices are
+// live, after compacting the live subgraph to local ids.
+template <bool TRI>
+__global__ void __launch_bounds__(1024, 1) peel_coop_kernel(const int64_t* __restrict__ ptr,
+                                                            const int32_t* __restrict__ adj,
+                                                            const int32_t* __restrict__ ta,
+                                                            const int32_t* __restrict__ tb,
+                                                            const int32_t* __restrict__ tc, uint8_t* tdead,
+                                                            int32_t* deg, int64_t* core, PeelChunk* Q0, PeelChunk* Q1,
+                                                            int32_t* A0, int32_t* A1, unsigned long long* ctrl,
+                                                            int64_t max_steps, int32_t solo, int32_t* slot,
+                                                            int32_t* coff, uint16_t* cadj) {
     cg::grid_group grid = cg::this_grid();
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     const int64_t warp = tid >> 5, nwarps = nthreads >> 5;
-    auto barrier = [&]() { grid.sync(); };
-    auto rd = [&](int i) -> unsigned long long { return __ldcg(ctrl + i); };
-    const int64_t* ptr = tri ? vptr : rowptr;
-    const int32_t* adj = tri ? vtri : col;
-    auto F = [&](int i) { return i ? F1 : F0; };
-    auto A = [&](int i) { return i ? A1 : A0; };
-    int cur = 0, a = 0;
-    int64_t k = 0, steps = 0;
+    int ph = 0, lv = 0;
+    int32_t k = 0;
+    int64_t steps = 0, na = (int64_t)__ldcg(ctrl + PC_LIST);
     for (;;) {
-        if (++steps > max_steps) {
-            if (tid == 0) ctrl[3] = 1;
-            return;
-        }
-        const int64_t na = (int64_t)rd(4 + a);
-        if (na <= solo) {
-            // peel_solo_kernel, launched next, finishes in one block
+        const int32_t* cl = lv & 1 ? A1 : A0;
+        int32_t* nlst = lv & 1 ? A0 : A1;
+        if constexpr (!TRI) if (na <= solo) {
+            __shared__ int32_t wsum[32];
+            for (int64_t i = tid; i < na; i += nthreads) {
+                const int32_t x = __ldcg(cl + i);
+                if (__ldcg(deg + x) >= 0) slot[x] = (int32_t)i;
+            }
+            if (blockIdx.x == 0) {
+                // row starts: a live vertex has deg live neighbours, padded to groups of 4
+                int32_t run = 0;
+                for (int64_t base = 0; base < na; base += blockDim.x) {
+                    const int64_t i = base + threadIdx.x;
+                    int32_t l = 0;
+                    if (i < na) l = (max(__ldcg(deg + __ldcg(cl + i)), 0) + 3) & ~3;
+                    int32_t incl = l;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += v;
+                    }
+                    if (lane == 31) wsum[threadIdx.x >> 5] = incl;
+                    __syncthreads();
+                    int32_t before = 0, tot = 0;
+                    for (int j = 0; j < (int)(blockDim.x >> 5); ++j) {
+                        if (j < (int)(threadIdx.x >> 5)) before += wsum[j];
+                        tot += wsum[j];
+                    }
+                    if (i < na) coff[i] = run + before + incl - l;
+                    run += tot;
+                    __syncthreads();
+                }
+                if (threadIdx.x == 0) coff[na] = run;
+            }
+            grid.sync();
+            for (int64_t i = warp; i < na; i += nwarps) {
+                const int32_t x = __ldcg(cl + i);
+                if (__ldcg(deg + x) < 0) continue;
+                int32_t o = __ldcg(coff + i);
+                const int32_t end = __ldcg(coff + i + 1);
+                const int64_t e = ptr[x + 1];
+                for (int64_t q0 = ptr[x]; q0 < e; q0 += 128) {
+                    int32_t y[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int64_t q = q0 + 32 * j + lane;
+                        y[j] = q < e ? adj[q] : -1;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) y[j] = y[j] >= 0 ? __ldcg(slot + y[j]) : -1;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const unsigned bal = __ballot_sync(0xffffffffu, y[j] >= 0);
+                        if (y[j] >= 0) cadj[o + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)y[j];
+                        o += __popc(bal);
+                    }
+                }
+                if (o + lane < end) cadj[o + lane] = 0xffff;
+            }
             if (tid == 0) {
-                ctrl[9] = (unsigned long long)a;
-                ctrl[10] = (unsigned long long)k;
-                ctrl[11] = (unsigned long long)(steps - 1);
-                ctrl[12] = 1;
+                ctrl[PC_SOLO + 1] = lv & 1;
+                ctrl[PC_SOLO + 2] = (unsigned long long)na;
+                ctrl[PC_SOLO + 3] = (unsigned long long)k;
+                ctrl[PC_SOLO + 4] = (unsigned long long)steps;
+                ctrl[PC_SOLO] = 1;
             }
             return;
         }
-        // level scan, warp by warp: one atomic per warp for each list and for the minimum
+        if (++steps > max_steps) {
+            if (tid == 0) ctrl[PC_ERR] = 1;
+            return;
+        }
+        if (tid == 0) {
+            ctrl[PC_Q + (ph + 2) % 3] = 0;
+            ctrl[PC_LIST + (lv + 2) % 3] = 0;
+            ctrl[PC_MIN + (lv + 1) % 3] = ~0ull;
+        }
+        unsigned long long* mnp = ctrl + PC_MIN + lv % 3;
+        // level scan, warp by warp: one atomic per warp for the list and for the minimum
         for (int64_t base = tid - lane; base < na; base += nthreads) {
             const int64_t i = base + lane;
-            int32_t x = -1, d = 0;
-            bool peel = false, keep = false;
+            int32_t x = 0, d = -1;
             if (i < na) {
-                x = __ldcg(A(a) + i);
-                if (__ldcg(alive + x)) {
-                    d = __ldcg(deg + x);
-                    peel = d <= k;
-                    keep = !peel;
-                }
+                x = __ldcg(cl + i);
+                d = __ldcg(deg + x);
             }
-            const unsigned pm = __ballot_sync(0xffffffffu, peel), km = __ballot_sync(0xffffffffu, keep);
+            const bool keep = d > k, peel = d >= 0 && d <= k;
+            const unsigned km = __ballot_sync(0xffffffffu, keep);
             const unsigned dmin = __reduce_min_sync(0xffffffffu, keep ? (unsigned)d : 0xffffffffu);
-            unsigned long long pb = 0, kb = 0;
-            if (lane == 0) {
-                if (pm) pb = atomicAdd(ctrl + cur, (unsigned long long)__popc(pm));
-                if (km) {
-                    kb = atomicAdd(ctrl + 5 - a, (unsigned long long)__popc(km));
-                    atomicMin(ctrl + 2, (unsigned long long)dmin);
-                }
+            unsigned long long kb = 0;
+            if (lane == 0 && km) {
+                kb = atomicAdd(ctrl + PC_LIST + (lv + 1) % 3, (unsigned long long)__popc(km));
+                if (dmin < __ldcg(mnp)) atomicMin(mnp, (unsigned long long)dmin);
             }
-            pb = __shfl_sync(0xffffffffu, pb, 0);
             kb = __shfl_sync(0xffffffffu, kb, 0);
-            const unsigned below = (1u << lane) - 1u;
+            if (keep) nlst[kb + __popc(km & ((1u << lane) - 1u))] = x;
             if (peel) {
-                alive[x] = 0;
+                deg[x] = PEEL_DEAD;
                 core[x] = k;
-                F(cur)[pb + __popc(pm & below)] = x;
             }
-            if (keep) A(1 - a)[kb + __popc(km & below)] = x;
+            peel_push(peel, x, ptr, (ph + 1) & 1 ? Q1 : Q0, ctrl + PC_Q + (ph + 1) % 3, lane);
         }
-        barrier();
-        unsigned long long f = rd(cur);
-        const unsigned long long kept = rd(5 - a);
-        const unsigned long long mn = rd(2);
-        barrier();
-        if (tid == 0) {
-            ctrl[4 + a] = 0;
-            ctrl[2] = ~0ull;
-        }
-        a = 1 - a;
-        if (f == 0) {
-            if (kept == 0) {
-                if (tid == 0) {
-                    ctrl[6] = (unsigned long long)steps;
-                    ctrl[7] = (unsigned long long)k;
-                }
-                return;
-            }
-            k = max(k + 1, (int64_t)mn);
-            barrier();
-            continue;
-        }
+        grid.sync();
+        ++ph;
+        int64_t nq = (int64_t)__ldcg(ctrl + PC_Q + ph % 3);
+        na = (int64_t)__ldcg(ctrl + PC_LIST + (lv + 1) % 3);
         // frontier rounds at level k
-        while (f > 0) {
+        while (nq > 0) {
             if (++steps > max_steps) {
-                if (tid == 0) ctrl[3] = 1;
+                if (tid == 0) ctrl[PC_ERR] = 1;
                 return;
             }
-            int32_t* fr = F(cur);
-            int32_t* nx = F(1 - cur);
-            unsigned long long* ncnt = ctrl + (1 - cur);
-            // light vertices by their lane; chunks of the heavy ones into the queue
-            for (int64_t base = warp * 32; base < (int64_t)f; base += nwarps * 32) {
-                const int64_t i = base + lane;
-                int32_t x = -1;
-                int64_t b = 0, len = 0;
-                if (i < (int64_t)f) {
-                    x = __ldcg(fr + i);
-                    b = ptr[x];
-                    len = ptr[x + 1] - b;
-                }
-                if (len <= PEEL_LIGHT) {
-                    int32_t it[PEEL_LIGHT];
-#pragma unroll
-                    for (int j = 0; j < PEEL_LIGHT; ++j) it[j] = j < len ? adj[b + j] : -1;
-#pragma unroll
-                    for (int j = 0; j < PEEL_LIGHT; ++j)
-                        if (it[j] >= 0) {
-                            if (tri) peel_triangle(it[j], x, k, ta, tb, tc, tdead, alive, deg, core, nx, ncnt);
-                            else peel_drop(it[j], k, alive, deg, core, nx, ncnt);
-                        }
-                }
-                const int32_t nch = len > PEEL_LIGHT ? (int32_t)((len + PEEL_CHUNK - 1) / PEEL_CHUNK) : 0;
-                int32_t incl = nch;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += v;
-                }
-                const int32_t tot = __shfl_sync(0xffffffffu, incl, 31);
-                unsigned long long cb = 0;
-                if (lane == 0 && tot) cb = atomicAdd(ctrl + 8, (unsigned long long)tot);
-                cb = __shfl_sync(0xffffffffu, cb, 0);
-                for (int32_t c = 0; c < nch; ++c) {
-                    const unsigned long long at = cb + (unsigned long long)(incl - nch + c);
-                    qv[at] = x;
-                    qs[at] = b + (int64_t)c * PEEL_CHUNK;
-                }
-            }
-            barrier();
-            const int64_t nq = (int64_t)rd(8);
+            if (tid == 0) ctrl[PC_Q + (ph + 2) % 3] = 0;
+            const PeelChunk* cq = ph & 1 ? Q1 : Q0;
+            PeelChunk* nx = (ph + 1) & 1 ? Q1 : Q0;
+            unsigned long long* ncnt = ctrl + PC_Q + (ph + 1) % 3;
+            unsigned mn = 0xffffffffu;
             for (int64_t c = warp; c < nq; c += nwarps) {
-                const int32_t x = __ldcg(qv + c);
-                const int64_t q0 = __ldcg(qs + c);
-                const int64_t q1 = min(q0 + (int64_t)PEEL_CHUNK, ptr[x + 1]);
-                int32_t it[PEEL_CHUNK / 32];
+                const int4 raw = __ldcg(reinterpret_cast<const int4*>(cq + c));
+                const int64_t q0 = (int64_t)(((unsigned long long)(unsigned)raw.y << 32) | (unsigned)raw.x);
+                const int32_t len = raw.z, x = raw.w;
+                int32_t it[2];
 #pragma unroll
-                for (int j = 0; j < PEEL_CHUNK / 32; ++j) {
-                    const int64_t q = q0 + lane + 32 * j;
-                    it[j] = q < q1 ? adj[q] : -1;
-                }
+                for (int j = 0; j < 2; ++j) it[j] = lane + 32 * j < len ? adj[q0 + lane + 32 * j] : -1;
+                if (!TRI) {
+                    bool hit[2];
 #pragma unroll
-                for (int j = 0; j < PEEL_CHUNK / 32; ++j)
-                    if (it[j] >= 0) {
-                        if (tri) peel_triangle(it[j], x, k, ta, tb, tc, tdead, alive, deg, core, nx, ncnt);
-                        else peel_drop(it[j], k, alive, deg, core, nx, ncnt);
+                    for (int j = 0; j < 2; ++j) {
+                        hit[j] = false;
+                        if (it[j] >= 0) {
+                            const int32_t old = atomicSub(deg + it[j], 1);
+                            hit[j] = old == k + 1;
+                            if (hit[j]) {
+                                deg[it[j]] = PEEL_DEAD;
+                                core[it[j]] = k;
+                            } else if (old > k) {
+                                mn = min(mn, (unsigned)(old - 1));
+                            }
+                        }
                     }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) peel_push(hit[j], it[j], ptr, nx, ncnt, lane);
+                } else {
+                    bool first[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        first[j] = false;
+                        if (it[j] >= 0) {
+                            unsigned int* word = (unsigned int*)(tdead + (it[j] & ~3));
+                            const unsigned int bit = 1u << (8 * (it[j] & 3));
+                            first[j] = !(atomicOr(word, bit) & bit);      // else it died with another vertex
+                        }
+                    }
+                    int32_t y[4];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        y[2 * j] = y[2 * j + 1] = -1;
+                        if (first[j]) {
+                            const int32_t a = ta[it[j]], b = tb[it[j]], cc = tc[it[j]];
+                            y[2 * j] = a == x ? b : a;
+                            y[2 * j + 1] = cc == x ? b : cc;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        // consecutive triangles of x share a member: one atomic per distinct vertex
+                        const unsigned peers = __match_any_sync(0xffffffffu, y[j]);
+                        bool hit = false;
+                        if (y[j] >= 0 && (peers & ((1u << lane) - 1u)) == 0) {
+                            const int32_t n = __popc(peers);
+                            const int32_t old = atomicSub(deg + y[j], n);
+                            hit = old > k && old - n <= k;
+                            if (hit) {
+                                deg[y[j]] = PEEL_DEAD;
+                                core[y[j]] = k;
+                            } else if (old > k) {
+                                mn = min(mn, (unsigned)(old - n));
+                            }
+                        }
+                        peel_push(hit, y[j], ptr, nx, ncnt, lane);
+                    }
+                }
             }
-            barrier();
-            f = rd(1 - cur);
-            barrier();
-            if (tid == 0) {
-                ctrl[cur] = 0;
-                ctrl[8] = 0;
+            if (warp < nq) {
+                mn = __reduce_min_sync(0xffffffffu, mn);
+                if (lane == 0 && mn < __ldcg(mnp)) atomicMin(mnp, (unsigned long long)mn);
             }
-            cur = 1 - cur;
-            barrier();
+            grid.sync();
+            ++ph;
+            nq = (int64_t)__ldcg(ctrl + PC_Q + ph % 3);
         }
-        k = k + 1;
+        const unsigned long long mb = __ldcg(mnp);
+        if (na == 0) {
+            if (tid == 0) {
+                ctrl[PC_STEPS] = (unsigned long long)steps;
+                ctrl[PC_LEVEL] = (unsigned long long)k;
+            }
+            return;
+        }
+        k = (int32_t)max((unsigned long long)k + 1, mb);
+        ++lv;
     }
 }
 
@@ -655,29 +775,41 @@ static void core_numbers_internal(lds_graph* g, bool tri, int64_t* core_int, con
     const int32_t nact = g->nact;
     const int blk = 256;
     if (nact == 0) return;
-    DevBuf<int32_t> deg(nact, s), frontier(nact, s);
     DevBuf<uint8_t> alive(nact, s);
     DevBuf<int32_t> nalive(1, s);
     LDS_CUDA(cudaMemsetAsync(nalive.get(), 0, sizeof(int32_t), s));
     LDS_LAUNCH(alive_init_kernel, grid_for(nact, blk), blk, 0, s, init_alive, nact, alive.get(), core_int, nalive.get());
+    if (tri) ensure_triangles(g);
+    int32_t remaining = nact;
+    if (init_alive) {
+        LDS_CUDA(cudaMemcpyAsync(&remaining, nalive.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        LDS_CUDA(cudaStreamSynchronize(s));
+    }
+    if (remaining == 0) return;
+    // every vertex alive: the whole graph's core numbers, peeled once per handle
+    DevBuf<int64_t>& whole = g->core_all[tri ? 1 : 0];
+    const bool all_alive = remaining == nact;
+    if (all_alive && whole.p) {
+        LDS_CUDA(cudaMemcpyAsync(core_int, whole.get(), (size_t)nact * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+        return;
+    }
+    DevBuf<int32_t> deg(nact, s);
     DevBuf<uint8_t> tdead;
-    LDS_CUDA(cudaMemsetAsync(deg.get(), 0, nact * sizeof(int32_t), s));
     // the triangle list the peeling walks: all of T, or, when few vertices are alive,
     // only the triangles whose three members are alive (the others never count)
     DevBuf<int32_t> cta, ctb, ctc, cvi;
     DevBuf<int64_t> cvp;
-    const int64_t* tvp = nullptr;
-    const int32_t *tvi = nullptr, *tta = nullptr, *ttb = nullptr, *ttc = nullptr;
+    const int64_t* ptr = g->rowptr.get();
+    const int32_t *adj = g->col.get(), *tta = nullptr, *ttb = nullptr, *ttc = nullptr;
     int64_t tnt = 0;
     if (!tri) {
-        LDS_LAUNCH(alive_degree_kernel, grid_for(nact, blk), blk, 0, s, g->rowptr.get(), g->col.get(), alive.get(), nact,
-                   deg.get());
+        if (all_alive)
+            LDS_LAUNCH(full_count_kernel, grid_for(nact, blk), blk, 0, s, ptr, alive.get(), nact, deg.get());
+        else
+            LDS_LAUNCH(alive_degree_kernel, grid_for((int64_t)nact * 32, blk), blk, 0, s, ptr, adj, alive.get(), nact,
+                       deg.get());
     } else {
-        ensure_triangles(g);
-        int32_t nal = 0;
-        LDS_CUDA(cudaMemcpyAsync(&nal, nalive.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        LDS_CUDA(cudaStreamSynchronize(s));
-        if (init_alive && (int64_t)nal * 4 < (int64_t)nact && g->ntri) {
+        if ((int64_t)remaining * 4 < (int64_t)nact && g->ntri) {
             const int64_t ntri = g->ntri;
             DevBuf<int32_t> flag(ntri + 1, s);
             DevBuf<int64_t> tpos(ntri + 1, s);
@@ -692,84 +824,61 @@ static void core_numbers_internal(lds_graph* g, bool tri, int64_t* core_int, con
                 LDS_LAUNCH(tri_compact_kernel, grid_for(ntri, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), ntri,
                            flag.get(), tpos.get(), cta.get(), ctb.get(), ctc.get());
             build_vertex_triangles(cta.get(), ctb.get(), ctc.get(), tnt, nact, cvp, cvi, s);
-            tvp = cvp.get();
-            tvi = cvi.get();
+            ptr = cvp.get();
+            adj = cvi.get();
             tta = cta.get();
             ttb = ctb.get();
             ttc = ctc.get();
         } else {
             ensure_vertex_triangles(g);
             tnt = g->ntri;
-            tvp = g->vt_ptr.get();
-            tvi = g->vt_idx.get();
+            ptr = g->vt_ptr.get();
+            adj = g->vt_idx.get();
             tta = g->ta.get();
             ttb = g->tb.get();
             ttc = g->tc.get();
         }
         tdead.alloc(((tnt + 3) & ~3ll) + 4, s);
         LDS_CUDA(cudaMemsetAsync(tdead.get(), 0, ((tnt + 3) & ~3ll) + 4, s));
-        if (tnt)
-            LDS_LAUNCH(alive_tri_count_kernel, grid_for(tnt, blk), blk, 0, s, tta, ttb, ttc, tnt, alive.get(), deg.get(),
-                       tdead.get());
+        if (all_alive || tta == cta.get()) {
+            // every triangle listed is live
+            LDS_LAUNCH(full_count_kernel, grid_for(nact, blk), blk, 0, s, ptr, alive.get(), nact, deg.get());
+        } else {
+            LDS_CUDA(cudaMemsetAsync(deg.get(), 0, nact * sizeof(int32_t), s));
+            if (tnt)
+                LDS_LAUNCH(alive_tri_count_kernel, grid_for(tnt, blk), blk, 0, s, tta, ttb, ttc, tnt, alive.get(),
+                           deg.get(), tdead.get());
+            LDS_LAUNCH(mark_dead_kernel, grid_for(nact, blk), blk, 0, s, alive.get(), nact, deg.get());
+        }
     }
-    int32_t remaining = 0;
-    LDS_CUDA(cudaMemcpyAsync(&remaining, nalive.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    LDS_CUDA(cudaStreamSynchronize(s));
-    if (remaining == 0) return;
-    // every vertex alive: the whole graph's core numbers, peeled once per handle
-    DevBuf<int64_t>& whole = g->core_all[tri ? 1 : 0];
-    const bool all_alive = remaining == nact;
-    if (all_alive && whole.p) {
-        LDS_CUDA(cudaMemcpyAsync(core_int, whole.get(), (size_t)nact * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-        return;
-    }
-    // one cooperative launch runs every level; the grid must be resident at once
-    DevBuf<unsigned long long> ctrl(13, s);
-    unsigned long long hctrl[13] = {0ull, 0ull, ~0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
+    DevBuf<unsigned long long> ctrl(PC_WORDS, s);
+    unsigned long long hctrl[PC_WORDS] = {};
+    for (int j = 0; j < 3; ++j) hctrl[PC_MIN + j] = ~0ull;
     LDS_CUDA(cudaMemcpyAsync(ctrl.get(), hctrl, sizeof(hctrl), cudaMemcpyHostToDevice, s));
-    DevBuf<int32_t> F1(nact, s), A0(nact, s), A1(nact, s);
-    // chunk queue: at most one chunk per vertex plus one per PEEL_CHUNK incidences
+    const int64_t max_steps = 4 * (int64_t)nact + 64;
+    // a small graph peels in one block from the start; a triangle peel only while its
+    // dead bits fit and its incidences do not need more than one SM
+    const bool small = nact <= PEEL_SOLO && (!tri || tnt <= PEEL_SOLO_TRIS);
     const int64_t incid = tri ? 3 * tnt : 2 * g->m;
-    const int64_t qcap = (int64_t)nact + incid / PEEL_CHUNK + 1;
-    DevBuf<int32_t> qv(qcap, s);
-    DevBuf<int64_t> qs(qcap, s);
-    LDS_LAUNCH(alive_list_kernel, grid_for(nact, blk), blk, 0, s, alive.get(), nact, A0.get(), ctrl.get() + 4);
-    // one block of 1024 threads per SM: grid barriers get cheaper with fewer blocks
-    const int pblk = 1024;
-    int per_sm = 0;
-    LDS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, peel_coop_kernel, pblk, 0));
-    LDS_CUDA(cudaFuncSetAttribute(peel_solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PEEL_SOLO_SMEM));
-    LDS_REQUIRE(per_sm > 0, LDS_ECUDA, "core numbers: peeling kernel cannot be resident");
-    int grid = std::max(1, std::min(num_sms(), (int)((nact + pblk - 1) / pblk)));
-    int64_t max_steps = 4 * (int64_t)nact + 64;
-    // the one-block tail only for edges: a triangle tail's incidences (hub
-    // triangles) keep the whole grid busy (R-MAT 20: 3.1 s instead of 5.9 s per
-    // LTDS query with the tail in one block)
-    int64_t solo = tri ? 0 : PEEL_SOLO;
-    DevBuf<int32_t> slotb(nact, s);
-    LDS_CUDA(cudaMemsetAsync(slotb.get(), 0xff, (size_t)nact * sizeof(int32_t), s));
-    int32_t* slp = slotb.get();
-    bool trib = tri;
-    const int64_t* rp = g->rowptr.get();
-    const int32_t* cl = g->col.get();
-    const int64_t* vp = tri ? tvp : nullptr;
-    const int32_t* vi = tri ? tvi : nullptr;
-    const int32_t* pa = tri ? tta : nullptr;
-    const int32_t* pb = tri ? ttb : nullptr;
-    const int32_t* pc = tri ? ttc : nullptr;
+    // a vertex is queued once: at most one chunk per vertex plus one per PEEL_CHUNK incidences
+    const int64_t qcap = small ? 0 : (int64_t)nact + incid / PEEL_CHUNK + 1;
+    const bool tail = !small && !tri;
+    DevBuf<PeelChunk> Q0(qcap, s), Q1(qcap, s);
+    DevBuf<int32_t> A0(small ? 0 : nact, s), A1(small ? 0 : nact, s);
+    // the one-block tail only for edges: a triangle tail's incidences (hub triangles)
+    // keep the whole grid busy
+    const int32_t solo = tri ? -1 : PEEL_SOLO;
+    DevBuf<int32_t> slotb(tail ? nact : 0, s), coff(tail ? PEEL_SOLO + 1 : 0, s);
+    // live neighbours of at most PEEL_SOLO vertices, rows padded to groups of 4
+    const int64_t ccap = std::min<int64_t>(2 * g->m, (int64_t)PEEL_SOLO * (PEEL_SOLO - 1)) + 4 * PEEL_SOLO;
+    DevBuf<uint16_t> cadj(tail ? ccap : 0, s);
     uint8_t* td = tri ? tdead.get() : nullptr;
-    uint8_t* al = alive.get();
     int32_t* dg = deg.get();
-    int32_t* f0 = frontier.get();
-    int32_t* f1 = F1.get();
-    int32_t* a0 = A0.get();
-    int32_t* a1 = A1.get();
+    PeelChunk *q0 = Q0.get(), *q1 = Q1.get();
+    int32_t *a0 = A0.get(), *a1 = A1.get();
     unsigned long long* ct = ctrl.get();
-    int32_t* qvp = qv.get();
-    int64_t* qsp = qs.get();
-    void* args[] = {(void*)&trib, (void*)&rp, (void*)&cl, (void*)&vp, (void*)&vi, (void*)&pa, (void*)&pb, (void*)&pc,
-                    (void*)&td, (void*)&al, (void*)&dg, (void*)&core_int, (void*)&f0, (void*)&f1, (void*)&a0,
-                    (void*)&a1, (void*)&qvp, (void*)&qsp, (void*)&ct, (void*)&max_steps, (void*)&solo};
+    int32_t *slp = slotb.get(), *cop = coff.get();
+    uint16_t* cap = cadj.get();
     const char* vb = getenv("LDS_VERBOSE");
     const bool verbose = vb && vb[0] == '1';
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -778,10 +887,36 @@ static void core_numbers_internal(lds_graph* g, bool tri, int64_t* core_int, con
         LDS_CUDA(cudaEventCreate(&e1));
         LDS_CUDA(cudaEventRecord(e0, s));
     }
-    LDS_CUDA(cudaLaunchCooperativeKernel((void*)peel_coop_kernel, dim3(grid), dim3(pblk), args, 0, s));
-    LDS_LAUNCH(peel_solo_kernel, 1, PEEL_SOLO_T, PEEL_SOLO_SMEM, s, trib, tri ? tvp : g->rowptr.get(),
-               tri ? tvi : g->col.get(), pa, pb, pc, td, al, dg, core_int, a0, a1, slp, ct, max_steps);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
+    int grid = 1;
+    if (small && tri) {
+        LDS_CUDA(cudaFuncSetAttribute(peel_solo_kernel<SOLO_TRIS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)PEEL_SOLO_TRIS_SMEM));
+        LDS_LAUNCH(peel_solo_kernel<SOLO_TRIS>, 1, PEEL_SOLO_T, PEEL_SOLO_TRIS_SMEM, s, a0, a1, dg, cop, cap, nact, ptr,
+                   adj, tta, ttb, ttc, td, tnt, core_int, ct, max_steps);
+    } else if (small) {
+        LDS_CUDA(cudaFuncSetAttribute(peel_solo_kernel<SOLO_EDGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)PEEL_SOLO_SMEM));
+        LDS_LAUNCH(peel_solo_kernel<SOLO_EDGES>, 1, PEEL_SOLO_T, PEEL_SOLO_SMEM, s, a0, a1, dg, cop, cap, nact, ptr, adj,
+                   tta, ttb, ttc, td, tnt, core_int, ct, max_steps);
+    } else {
+        LDS_LAUNCH(alive_list_kernel, grid_for(nact, blk), blk, 0, s, alive.get(), nact, a0, ct + PC_LIST);
+        // one block of 1024 threads per SM: grid barriers get cheaper with fewer blocks
+        const int pblk = 1024;
+        const void* fn = tri ? (const void*)peel_coop_kernel<true> : (const void*)peel_coop_kernel<false>;
+        grid = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms(), ((int64_t)nact + incid / 8 + pblk - 1) / pblk));
+        if (tail) LDS_CUDA(cudaMemsetAsync(slotb.get(), 0xff, (size_t)nact * sizeof(int32_t), s));
+        void* args[] = {(void*)&ptr, (void*)&adj, (void*)&tta, (void*)&ttb, (void*)&ttc, (void*)&td, (void*)&dg,
+                        (void*)&core_int, (void*)&q0, (void*)&q1, (void*)&a0, (void*)&a1, (void*)&ct,
+                        (void*)&max_steps, (void*)&solo, (void*)&slp, (void*)&cop, (void*)&cap};
+        LDS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(pblk), args, 0, s));
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        if (tail) {
+            LDS_CUDA(cudaFuncSetAttribute(peel_solo_kernel<SOLO_TAIL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)PEEL_SOLO_SMEM));
+            LDS_LAUNCH(peel_solo_kernel<SOLO_TAIL>, 1, PEEL_SOLO_T, PEEL_SOLO_SMEM, s, a0, a1, dg, cop, cap, nact, ptr,
+                       adj, tta, ttb, ttc, td, tnt, core_int, ct, max_steps);
+        }
+    }
     if (verbose) LDS_CUDA(cudaEventRecord(e1, s));
     LDS_CUDA(cudaMemcpyAsync(hctrl, ctrl.get(), sizeof(hctrl), cudaMemcpyDeviceToHost, s));
     LDS_CUDA(cudaStreamSynchronize(s));
@@ -789,11 +924,11 @@ static void core_numbers_internal(lds_graph* g, bool tri, int64_t* core_int, con
         float ms = 0;
         cudaEventElapsedTime(&ms, e0, e1);
         fprintf(stderr, "[core] nact=%d live=%d peel %.2f ms, %llu steps, last level %llu, grid %d\n", nact, remaining,
-                ms, hctrl[6], hctrl[7], grid);
+                ms, hctrl[PC_STEPS], hctrl[PC_LEVEL], grid);
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
     }
-    LDS_REQUIRE(hctrl[3] == 0, LDS_ETIMEOUT, "core numbers: peeling hit its iteration bound");
+    LDS_REQUIRE(hctrl[PC_ERR] == 0, LDS_ETIMEOUT, "core numbers: peeling hit its iteration bound");
     if (all_alive) {
         whole.alloc(nact, s);
         LDS_CUDA(cudaMemcpyAsync(whole.get(), core_int, (size_t)nact * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
