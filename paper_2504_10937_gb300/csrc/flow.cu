@@ -324,18 +324,42 @@ struct HNet {
     int64_t* tcap;         // [nv] residual capacity to t
     int64_t* excess;       // [nv]
     int32_t* h;            // [nv] exact distance to t (DEAD: cannot reach it)
+    int64_t* claim;        // [nv] admissible capacity claimed in this sweep
+    const int2* chunk;     // vertex and first incidence of every chunk of HY_CHUNK incidences
+    const int64_t* nchunk; // their number
 };
 
-// widths above 3 are refused; count[v] = incidences of v; in[v] = flow v receives
+constexpr int HY_GROUP = 8;                    // lanes that take a chunk together
+constexpr int HY_ITEMS = 4;                    // incidences per lane
+constexpr int HY_CHUNK = HY_GROUP * HY_ITEMS;
+constexpr int HY_THREADS = 1024;
+
+__global__ void hyper_chunk_count_kernel(const int64_t* vptr, int32_t nv, int32_t* cnt) {
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= nv; v += stride)
+        cnt[v] = v < nv ? (int32_t)((vptr[v + 1] - vptr[v] + HY_CHUNK - 1) / HY_CHUNK) : 0;
+}
+
+// one warp per vertex
+__global__ void hyper_chunk_fill_kernel(const int64_t* vptr, int32_t nv, const int64_t* coff, int2* chunk) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < nv; v += nwarps)
+        for (int64_t c = coff[v] + lane; c < coff[v + 1]; c += 32)
+            chunk[c] = make_int2((int32_t)v, (int32_t)(vptr[v] + (c - coff[v]) * HY_CHUNK));
+}
+
+// widths above 3 are refused (wide bit 0; bit 1: some pattern has three members); count[v] = incidences of v; in[v] = flow v receives
 __global__ void hyper_degree_kernel(const int64_t* pptr, const int32_t* pidx, int32_t np, const int64_t* f,
                                     int32_t* deg, ull* in, int32_t* wide) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < np; j += stride) {
         const int64_t b = pptr[j], e = pptr[j + 1], len = e - b;
         if (len > 3) {
-            *wide = 1;
+            atomicOr(wide, 1);
             continue;
         }
+        if (len == 3 && !(__ldcg(wide) & 2)) atomicOr(wide, 2);
         for (int64_t k = b; k < e; ++k) {
             atomicAdd(in + pidx[k], (ull)f[k]);
             if (len >= 2) atomicAdd(deg + pidx[k], 1);
@@ -388,170 +412,252 @@ __global__ void hyper_init_kernel(HNet net, const ull* in, int64_t pK, ull* flow
 
 // hyper_flow_kernel control words
 enum : int {
-    HC_LEVEL = 0,      // [0..2] vertices labelled per breadth-first level (three rotating counters)
-    HC_ACTIVE = 3,     // vertices with excess and a label
-    HC_STUCK = 4,      // vertices with excess and no path to t
-    HC_LMAX = 5,       // highest label holding excess
-    HC_FLOW = 6,       // flow into t
-    HC_STATUS = 7,     // 0 finished, 1 phase bound hit, 2 stopped: some excess cannot reach t
-    HC_PHASES = 8,
-    HC_LEVELS = 9,     // breadth-first levels run in all
-    HC_WORDS = 10
+    HC_EXCESS = 0,     // [3] vertices holding excess (by phase, three rotating counters)
+    HC_ACTIVE = 3,     // [3] of them, those that label 1 takes
+    HC_ADDED = 6,      // [3] a breadth-first level: vertices it labelled, << 32 those holding excess
+    HC_FLOW = 9,       // flow into t
+    HC_STATUS = 10,    // 0 finished, 1 phase bound hit, 2 stopped: some excess cannot reach t
+    HC_PHASES = 11,
+    HC_LEVELS = 12,    // breadth-first levels run in all
+    HC_WORDS = 13
 };
 
-// One cooperative launch runs the whole preflow phase.  Each phase computes
-// exact distance labels by a breadth-first search from t over the residual
-// hyper-arcs (a global relabel), then sweeps the labels from the highest one
-// that holds excess down to 1: every vertex at label L with excess pushes it
-// along its admissible hyper-arcs (to members at label L - 1), in incidence
-// order, until the excess or those arcs run out; vertices at label 1 push into
-// t.  Within a label no two vertices touch the same share from below (a share
-// is lowered only by its own vertex, and vertices at label L receive nothing
-// while label L is swept), so a push needs atomics only on the target's share
-// and excess.  After the sweep every vertex that still holds excess has no
-// admissible hyper-arc, and since no push shortens a distance, its label rises
-// in the next phase; labels are at most nv, so there are at most nv^2 + 1
-// phases.  One warp serves one vertex; `max_phases` bounds the loop (status 1).
-__global__ void __launch_bounds__(FB) hyper_flow_kernel(HNet net, ull* ctrl, int64_t max_phases, int stop_if_short) {
+// One cooperative launch runs the whole preflow phase.  Each phase settles the
+// vertices (what the last sweep pushed leaves their excess; label 1 pushes into t),
+// computes exact distance labels by a breadth-first search from t over the residual
+// hyper-arcs (a global relabel), stopping once every vertex that holds excess has a
+// label, then sweeps the labels from the highest down to 2: every vertex at label L
+// with excess pushes it along its admissible hyper-arcs (to members at label L - 1)
+// until the excess or those arcs run out.  Within a label no two vertices touch the
+// same share from below (a share is lowered only by its own vertex, and vertices at
+// label L receive nothing while label L is swept), so a push needs atomics only on
+// the target's share and excess.  The chunks of one vertex share its excess through
+// `claim`: a chunk adds its admissible capacity there and may push what of the
+// excess lies past the capacity claimed before it, so exactly min(excess, admissible
+// capacity) leaves the vertex.  Every vertex that still holds excess then has no
+// admissible hyper-arc, and since no push shortens a distance, its label rises in
+// the next phase; labels are at most nv, so there are at most nv^2 + 1 phases.
+// `max_phases` bounds the loop (status 1).
+//
+// The phases are short and many (100 on the 1,511-vertex core of the 1M-vertex
+// power-law graph), so what bounds a step is its chain of L2 accesses and the grid
+// barrier.  Incidences are cut into chunks of 32, eight lanes take one with four
+// loads in flight each, and a lane looks at one chunk's vertex to find the chunks
+// that have work, so low and high degrees spread alike; one block of 1,024 threads
+// per SM keeps the barrier cheap.  IsDensest, building the network included, against
+// one warp per vertex and four blocks per SM (GB300): that core 7.3 -> 3.0 ms; 37,622
+// vertices of degree 11 (Barabasi-Albert) 9.4 -> 1.4 ms; 66.6M incidences of 988
+// vertices (R-MAT scale 18 triangles) 90 -> 55 ms.
+template <bool PAIRS>
+__global__ void __launch_bounds__(HY_THREADS, 1) hyper_flow_kernel(const HNet net, ull* ctrl, int64_t max_phases,
+                                                                   int stop_if_short, int want_side) {
     cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = tid >> 5, nwarps = nthreads >> 5;
+    const int lane = threadIdx.x & 31, gl = lane & (HY_GROUP - 1), gbase = lane & ~(HY_GROUP - 1);
+    const int64_t warp = tid >> 5, ngroups = nthreads / HY_GROUP;
     const int32_t nv = net.nv;
+    const int64_t nc = *net.nchunk;
+    // calls body(active, v, start, e) warp-wide for every chunk that pick(v, e) takes,
+    // one per group of lanes at a time; e is what pick stored
+    auto for_chunks = [&](auto&& pick, auto&& body) {
+        for (int64_t base = warp * (32 / HY_GROUP); base < nc; base += HY_GROUP * ngroups) {
+            const int64_t c = base + gbase / HY_GROUP + (int64_t)gl * ngroups;
+            int2 ch = make_int2(0, 0);
+            int64_t e = 0;
+            bool take = false;
+            if (c < nc) {
+                ch = net.chunk[c];
+                take = pick(ch.x, e);
+            }
+            unsigned mask = (__ballot_sync(FULL, take) >> gbase) & ((1u << HY_GROUP) - 1u);
+            while (__any_sync(FULL, mask != 0)) {
+                const bool on = mask != 0;
+                const int from = gbase + (on ? __ffs(mask) - 1 : 0);
+                mask &= mask - 1;
+                const int32_t v = __shfl_sync(FULL, ch.x, from), st = __shfl_sync(FULL, ch.y, from);
+                body(on, v, st, __shfl_sync(FULL, e, from));
+            }
+        }
+    };
+    int lc = 0;                                   // breadth-first levels so far
     for (int64_t phase = 0;; ++phase) {
         if (phase >= max_phases) {
             if (tid == 0) ctrl[HC_STATUS] = 1;
             return;
         }
+        const int ps = (int)(phase % 3), pn = (int)((phase + 1) % 3);
         if (tid == 0) {
-            ctrl[HC_LEVEL] = ctrl[HC_LEVEL + 1] = ctrl[HC_LEVEL + 2] = 0;
-            ctrl[HC_ACTIVE] = ctrl[HC_STUCK] = ctrl[HC_LMAX] = 0;
+            ctrl[HC_EXCESS + pn] = ctrl[HC_ACTIVE + pn] = 0;
+            ctrl[HC_ADDED + lc % 3] = 0;
             ctrl[HC_PHASES] = (ull)phase + 1;
         }
-        for (int64_t v = tid; v < nv; v += nthreads) net.h[v] = __ldcg(net.tcap + v) > 0 ? 1 : DEAD;
+        // settle: excess after the last sweep, label 1 for what can still push into t
+        {
+            unsigned ne = 0, na = 0;
+            ull fl = 0;
+            for (int64_t v = tid; v < nv; v += nthreads) {
+                int64_t e = __ldcg(net.excess + v), tc = __ldcg(net.tcap + v);
+                if (phase > 0 && e > 0) {
+                    if (__ldcg(net.h + v) == 1) {
+                        const int64_t d = min(e, tc);
+                        tc -= d;
+                        e -= d;
+                        fl += (ull)d;
+                        net.tcap[v] = tc;
+                        net.excess[v] = e;
+                    } else {
+                        const int64_t d = min(e, __ldcg(net.claim + v));
+                        if (d) {
+                            e -= d;
+                            net.excess[v] = e;
+                            net.claim[v] = 0;
+                        }
+                    }
+                }
+                net.h[v] = tc > 0 ? 1 : DEAD;
+                ne += e > 0;
+                na += e > 0 && tc > 0;
+            }
+            ne = __reduce_add_sync(FULL, ne);
+            na = __reduce_add_sync(FULL, na);
+            for (int o = 16; o; o >>= 1) fl += __shfl_xor_sync(FULL, fl, o);
+            if (lane == 0) {
+                if (ne) atomicAdd(ctrl + HC_EXCESS + ps, (ull)ne);
+                if (na) atomicAdd(ctrl + HC_ACTIVE + ps, (ull)na);
+                if (fl) atomicAdd(ctrl + HC_FLOW, fl);
+            }
+        }
         grid.sync();
+        const ull ne = __ldcg(ctrl + HC_EXCESS + ps);
+        ull act = __ldcg(ctrl + HC_ACTIVE + ps);
+        if (ne == 0 && !want_side) return;               // the flow is complete (status 0)
         // breadth-first levels: an unlabelled vertex joins level L + 1 when one of its
         // hyper-arcs (share > 0) leads to a member at level L
-        for (int32_t L = 1;; ++L) {
-            for (int64_t v = warp; v < nv; v += nwarps) {
-                if (__ldcg(net.h + v) != DEAD) continue;
-                const int64_t b0 = net.vptr[v], b1 = net.vptr[v + 1];
-                bool found = false;
-                for (int64_t base = b0; base < b1 && !found; base += 32) {
-                    const int64_t i = base + lane;
-                    bool hit = false;
-                    if (i < b1 && __ldcg(net.f + i) > 0) {
-                        const int32_t a = net.w1[i], c = net.w2[i];
-                        hit = (a >= 0 && __ldcg(net.h + a) == L) || (c >= 0 && __ldcg(net.h + c) == L);
-                    }
-                    found = __any_sync(FULL, hit);
-                }
-                if (found && lane == 0) {
-                    net.h[v] = L + 1;
-                    atomicAdd(ctrl + HC_LEVEL + (L % 3), 1ull);
-                }
-            }
-            grid.sync();
-            const ull added = __ldcg(ctrl + HC_LEVEL + (L % 3));
+        int32_t top = 1;
+        while (ne == 0 || act < ne) {
+            const int32_t L = top;
             if (tid == 0) {
-                ctrl[HC_LEVEL + ((L + 2) % 3)] = 0;
+                ctrl[HC_ADDED + (lc + 1) % 3] = 0;
                 ctrl[HC_LEVELS] += 1;
             }
-            if (added == 0) break;
+            unsigned won = 0, wone = 0;                  // vertices this thread labelled, those holding excess
+            for_chunks([&](int32_t v, int64_t&) { return __ldcg(net.h + v) == DEAD; },
+                       [&](bool on, int32_t v, int32_t st, int64_t) {
+                           bool hit = false;
+                           if (on) {
+                               const int32_t end = (int32_t)min(net.vptr[v + 1], (int64_t)st + HY_CHUNK);
+                               int32_t w[HY_ITEMS][2];
+#pragma unroll
+                               for (int j = 0; j < HY_ITEMS; ++j) {
+                                   const int32_t i = st + gl + j * HY_GROUP;
+                                   w[j][0] = w[j][1] = -1;
+                                   if (i < end && __ldcg(net.f + i) > 0) {
+                                       w[j][0] = net.w1[i];
+                                       if (!PAIRS) w[j][1] = net.w2[i];
+                                   }
+                               }
+#pragma unroll
+                               for (int j = 0; j < HY_ITEMS; ++j) {
+                                   if (w[j][0] >= 0) hit |= __ldcg(net.h + w[j][0]) == L;
+                                   if (!PAIRS && w[j][1] >= 0) hit |= __ldcg(net.h + w[j][1]) == L;
+                               }
+                           }
+                           const unsigned any = (__ballot_sync(FULL, hit) >> gbase) & ((1u << HY_GROUP) - 1u);
+                           // the group's first lane labels the vertex, once
+                           if (any && gl == 0 && atomicCAS(net.h + v, DEAD, L + 1) == DEAD) {
+                               ++won;
+                               wone += __ldcg(net.excess + v) > 0;
+                           }
+                       });
+            won = __reduce_add_sync(FULL, won);
+            wone = __reduce_add_sync(FULL, wone);
+            if (lane == 0 && won) atomicAdd(ctrl + HC_ADDED + lc % 3, ((ull)wone << 32) | won);
+            grid.sync();
+            // this level's own counter: blocks that run ahead write the next one
+            const ull added = __ldcg(ctrl + HC_ADDED + lc % 3);
+            act += added >> 32;
+            ++lc;
+            if (!added) break;
+            top = L + 1;
         }
-        // vertices holding excess: with a label (active) or without (stuck)
-        {
-            ull act = 0, stk = 0;
-            int32_t lmax = 0;
-            for (int64_t v = tid; v < nv; v += nthreads) {
-                if (__ldcg(net.excess + v) > 0) {
-                    const int32_t hv = __ldcg(net.h + v);
-                    if (hv < DEAD) {
-                        ++act;
-                        lmax = max(lmax, hv);
-                    } else {
-                        ++stk;
-                    }
-                }
-            }
-            for (int o = 16; o; o >>= 1) {
-                act += __shfl_xor_sync(FULL, act, o);
-                stk += __shfl_xor_sync(FULL, stk, o);
-                lmax = max(lmax, __shfl_xor_sync(FULL, lmax, o));
-            }
-            if (lane == 0) {
-                if (act) atomicAdd(ctrl + HC_ACTIVE, act);
-                if (stk) atomicAdd(ctrl + HC_STUCK, stk);
-                if (lmax) atomicMax(ctrl + HC_LMAX, (ull)lmax);
-            }
-        }
-        grid.sync();
-        const ull act = __ldcg(ctrl + HC_ACTIVE), stk = __ldcg(ctrl + HC_STUCK);
-        const int32_t lmax = (int32_t)__ldcg(ctrl + HC_LMAX);
-        if (stop_if_short && stk > 0) {
+        if (ne == 0) return;
+        if (stop_if_short && act < ne) {
             if (tid == 0) ctrl[HC_STATUS] = 2;
             return;
         }
-        if (act == 0) {
-            if (tid == 0) ctrl[HC_STATUS] = 0;
-            return;
-        }
+        if (act == 0) return;
         // downhill sweep
-        for (int32_t L = lmax; L >= 1; --L) {
-            for (int64_t v = warp; v < nv; v += nwarps) {
-                if (__ldcg(net.h + v) != L) continue;
-                const int64_t e = __ldcg(net.excess + v);
-                if (e <= 0) continue;
-                if (L == 1) {
-                    if (lane == 0) {
-                        const int64_t tc = __ldcg(net.tcap + v);
-                        const int64_t d = min(e, tc);
-                        if (d > 0) {
-                            net.tcap[v] = tc - d;
-                            net.excess[v] = e - d;
-                            atomicAdd(ctrl + HC_FLOW, (ull)d);
-                        }
+        for (int32_t L = top; L >= 2; --L) {
+            for_chunks(
+                [&](int32_t v, int64_t& e) {
+                    if (__ldcg(net.h + v) != L) return false;
+                    e = __ldcg(net.excess + v);
+                    return e > 0;
+                },
+                [&](bool on, int32_t v, int32_t st, int64_t e) {
+                    int64_t cap[HY_ITEMS], mine = 0;
+                    int32_t to[HY_ITEMS];
+                    bool second[HY_ITEMS];
+#pragma unroll
+                    for (int j = 0; j < HY_ITEMS; ++j) {
+                        cap[j] = 0;
+                        to[j] = -1;
+                        second[j] = false;
                     }
-                    continue;
-                }
-                const int64_t b0 = net.vptr[v], b1 = net.vptr[v + 1];
-                int64_t rem = e;
-                for (int64_t base = b0; base < b1 && rem > 0; base += 32) {
-                    const int64_t i = base + lane;
-                    int64_t cap = 0;
-                    int32_t to_i = -1, to_v = -1;
-                    if (i < b1) {
-                        const int64_t fi = __ldcg(net.f + i);
-                        if (fi > 0) {
-                            const int32_t a = net.w1[i], c = net.w2[i];
-                            if (a >= 0 && __ldcg(net.h + a) == L - 1) {
-                                cap = fi;
-                                to_i = net.o1[i];
-                                to_v = a;
-                            } else if (c >= 0 && __ldcg(net.h + c) == L - 1) {
-                                cap = fi;
-                                to_i = net.o2[i];
-                                to_v = c;
+                    if (on) {
+                        const int32_t end = (int32_t)min(net.vptr[v + 1], (int64_t)st + HY_CHUNK);
+                        int32_t w[HY_ITEMS][2];
+#pragma unroll
+                        for (int j = 0; j < HY_ITEMS; ++j) {
+                            const int32_t i = st + gl + j * HY_GROUP;
+                            w[j][0] = w[j][1] = -1;
+                            if (i < end) {
+                                cap[j] = __ldcg(net.f + i);
+                                w[j][0] = net.w1[i];
+                                if (!PAIRS) w[j][1] = net.w2[i];
                             }
+                        }
+#pragma unroll
+                        for (int j = 0; j < HY_ITEMS; ++j) {
+                            if (cap[j] > 0) {
+                                if (w[j][0] >= 0 && __ldcg(net.h + w[j][0]) == L - 1) {
+                                    to[j] = w[j][0];
+                                } else if (!PAIRS && w[j][1] >= 0 && __ldcg(net.h + w[j][1]) == L - 1) {
+                                    to[j] = w[j][1];
+                                    second[j] = true;
+                                }
+                            }
+                            if (to[j] < 0) cap[j] = 0;
+                            mine += cap[j];
                         }
                     }
                     // shares of all incidences sum to at most np q K <= 2^61: no overflow
-                    int64_t incl = cap;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int64_t t = __shfl_up_sync(FULL, incl, o);
-                        if (lane >= o) incl += t;
+                    int64_t incl = mine;
+#pragma unroll
+                    for (int o = 1; o < HY_GROUP; o <<= 1) {
+                        const int64_t t = __shfl_up_sync(FULL, incl, o, HY_GROUP);
+                        if (gl >= o) incl += t;
                     }
-                    const int64_t d = max((int64_t)0, min(cap, rem - (incl - cap)));
-                    if (d > 0) {
-                        net.f[i] -= d;
-                        atomicAdd((ull*)(net.f + to_i), (ull)d);
-                        atomicAdd((ull*)(net.excess + to_v), (ull)d);
+                    const int64_t all = __shfl_sync(FULL, incl, HY_GROUP - 1, HY_GROUP);
+                    int64_t before = 0;
+                    if (gl == 0 && all > 0) before = (int64_t)atomicAdd((ull*)(net.claim + v), (ull)all);
+                    before = __shfl_sync(FULL, before, 0, HY_GROUP);
+                    if (all > 0) {
+                        int64_t rem = e - before - (incl - mine);       // excess left for this lane's arcs
+#pragma unroll
+                        for (int j = 0; j < HY_ITEMS; ++j) {
+                            const int64_t d = min(cap[j], rem);
+                            if (d > 0) {
+                                const int32_t i = st + gl + j * HY_GROUP;
+                                __stcg(net.f + i, cap[j] - d);
+                                atomicAdd((ull*)(net.f + (second[j] ? net.o2[i] : net.o1[i])), (ull)d);
+                                atomicAdd((ull*)(net.excess + to[j]), (ull)d);
+                            }
+                            rem -= cap[j];
+                        }
                     }
-                    rem -= min(rem, __shfl_sync(FULL, incl, 31));
-                }
-                if (lane == 0 && rem != e) net.excess[v] = rem;
-            }
+                });
             grid.sync();
         }
     }
@@ -581,31 +687,40 @@ static int64_t hyper_max_flow(const int64_t* pptr, const int32_t* pidx, int32_t 
     int32_t hwide = 0;
     LDS_CUDA(cudaMemcpyAsync(&hwide, wide.get(), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     LDS_CUDA(cudaStreamSynchronize(s));
-    LDS_REQUIRE(hwide == 0, LDS_EINVAL, "max flow: a pattern has more than three members");
+    LDS_REQUIRE(!(hwide & 1), LDS_EINVAL, "max flow: a pattern has more than three members");
     LDS_REQUIRE(ninc < (int64_t)INT32_MAX, LDS_EOVERFLOW, "max flow: %lld incidences exceed the 32-bit index",
                 (long long)ninc);
     DevBuf<int32_t> pos(std::max<int64_t>(nidx, 1), s);
     DevBuf<int64_t> f(std::max<int64_t>(ninc, 1), s), tcap(nvp, s), excess(nvp, s);
     DevBuf<int32_t> o1(std::max<int64_t>(ninc, 1), s), o2(std::max<int64_t>(ninc, 1), s);
     DevBuf<int32_t> w1(std::max<int64_t>(ninc, 1), s), w2(std::max<int64_t>(ninc, 1), s), h(nvp, s);
-    HNet net{nv, vptr.get(), f.get(), o1.get(), o2.get(), w1.get(), w2.get(), tcap.get(), excess.get(), h.get()};
+    DevBuf<int64_t> claim(nvp, s), coff(nvp + 1, s);
+    DevBuf<int2> chunk((size_t)nvp + ninc / HY_CHUNK + 1, s);
+    LDS_CUDA(cudaMemsetAsync(claim.get(), 0, nvp * sizeof(int64_t), s));
+    HNet net{nv,         vptr.get(),   f.get(), o1.get(),    o2.get(),    w1.get(),       w2.get(),
+             tcap.get(), excess.get(), h.get(), claim.get(), chunk.get(), coff.get() + nv};
+    if (nv) {
+        DevBuf<int32_t> ccnt(nvp + 1, s);
+        LDS_LAUNCH(hyper_chunk_count_kernel, grid_for(nv + 1, FB), FB, 0, s, vptr.get(), nv, ccnt.get());
+        exclusive_scan_i32_dev(ccnt.get(), coff.get(), (int64_t)nv + 1, s);
+        LDS_LAUNCH(hyper_chunk_fill_kernel, grid_for((int64_t)nv * 32, FB), FB, 0, s, vptr.get(), nv, coff.get(),
+                   chunk.get());
+    }
     if (np) {
         LDS_LAUNCH(hyper_pos_kernel, grid_for(np, FB), FB, 0, s, pptr, pidx, np, vptr.get(), cursor.get(), pos.get());
         LDS_LAUNCH(hyper_fill_kernel, grid_for(np, FB), FB, 0, s, pptr, pidx, np, fslot, pos.get(), net);
     }
     if (nv) LDS_LAUNCH(hyper_init_kernel, grid_for(nv, FB), FB, 0, s, net, in.get(), pK, ctrl.get() + HC_FLOW);
     if (nv) {
-        int per_sm = 0;
-        LDS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hyper_flow_kernel, FB, 0));
-        LDS_REQUIRE(per_sm > 0, LDS_ECUDA, "max flow: the flow kernel cannot be resident");
-        // one warp per vertex; no more blocks than can be resident at once
-        const int64_t want = ((int64_t)nv * 32 + FB - 1) / FB;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms() * std::min(per_sm, 4)));
+        // a group of lanes per chunk; at most one block per SM, all resident at once
+        const int64_t want = (((int64_t)nv + ninc / HY_CHUNK) * HY_GROUP + HY_THREADS - 1) / HY_THREADS;
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, num_sms()));
         const int64_t max_phases = std::min<int64_t>((int64_t)nv * nv + 2, (int64_t)1 << 40);
-        int stop = stop_if_short ? 1 : 0;
+        int stop = stop_if_short ? 1 : 0, ws = side ? 1 : 0;
         ull* cp = ctrl.get();
-        void* args[] = {(void*)&net, (void*)&cp, (void*)&max_phases, (void*)&stop};
-        LDS_CUDA(cudaLaunchCooperativeKernel((void*)hyper_flow_kernel, dim3(grid), dim3(FB), args, 0, s));
+        void* args[] = {(void*)&net, (void*)&cp, (void*)&max_phases, (void*)&stop, (void*)&ws};
+        const void* fn = hwide & 2 ? (const void*)hyper_flow_kernel<false> : (const void*)hyper_flow_kernel<true>;
+        LDS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(HY_THREADS), args, 0, s));
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
     ull hc[HC_WORDS];
