@@ -382,12 +382,13 @@ lds_status lds_batch_autotune(int32_t count, const lds_query* queries, int32_t* 
 int32_t lds_debug_pick_next(int32_t nq, const int64_t* bytes, const uint8_t* graph_busy, int64_t free_bytes);
 
 /* Edge-density kernel choice for LDS_EXACT / LDS_FP32 (process-wide):
- *   0  automatic: a graph whose active vertices fit in shared memory (at
- *      most 24,576, every scaled load below 2^32) and with few edges (at most
- *      49,152) runs on one thread-block
- *      cluster of 8 CTAs, each holding every load word and 1/8 of the edges,
- *      the counts reduced and the new loads broadcast through distributed
- *      shared memory; otherwise the degree-oriented pass (each edge once, stored at its
+ *   0  automatic: a graph of at most 65,536 active vertices whose symmetric
+ *      CSR slots fit the chip's registers (up to 16,384 per CTA, rows whole;
+ *      the load words in shared memory, at most 57,344 vertices; every weight
+ *      and exact load below 2^32) runs with its slots resident, each endpoint
+ *      deciding its own edges, one barrier per iteration over one CTA, a
+ *      cluster of 8 or up to one CTA per SM; otherwise the degree-oriented
+ *      pass (each edge once, stored at its
  *      lower-degree endpoint, hot loads in shared memory) with 32-bit load
  *      words when every scaled load fits 32 bits, else with 64-bit keys
  *      (load, id), else variant 1.  With 32-bit words the pass counts only
@@ -401,9 +402,8 @@ int32_t lds_debug_pick_next(int32_t nq, const int64_t* bytes, const uint8_t* gra
  *      pass, one pass launch and one update launch per iteration;
  *   4  as 0 with 32-bit words, one pass launch and one update launch per
  *      iteration;
- *   5  as 0 without the cluster form (the cooperative launch for every size);
- *   6  as 0 with the cluster form for every graph that fits, whatever its
- *      edge count.
+ *   5  as 0 without the resident form (the cooperative launch for every size);
+ *   6  as 0 (kept for callers of the former cluster form).
  * All compute the same iterates.  Errors: LDS_EINVAL. */
 lds_status lds_set_fw_variant(int32_t variant);
 

@@ -662,20 +662,20 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
     if (d == LDS_EDGE) {
         EdgeFwOut fo;
         LDS_CUDA(cudaEventRecord(e0, s));
-        // graphs whose active vertices fit in shared memory run on one thread-block cluster
-        bool clus = false;
+        // graphs whose slots fit the chip's registers
+        bool res = false;
         if ((g_fw_variant == 0 || g_fw_variant == 6) && (p == LDS_EXACT || p == LDS_FP32)) {
             if (want_last) g->fw_last.alloc(std::max<int64_t>(g->m, 1), s);
             timer.start(s);
-            clus = fw_cluster_run(g, iters, p, want_last ? g->fw_last.get() : nullptr, g_fw_variant == 6);
-            if (clus) timer.stop(s, iters);
+            res = fw_resident_run(g, iters, p, want_last ? g->fw_last.get() : nullptr);
+            if (res) timer.stop(s, iters);
             else g->fw_last.release();
         }
-        bool fast = !clus && g_fw_variant != 1 && run_edge_fw_oriented(g, iters, p, true, want_last, fo, timer);
-        if (clus) {
+        bool fast = !res && g_fw_variant != 1 && run_edge_fw_oriented(g, iters, p, true, want_last, fo, timer);
+        if (res) {
             LDS_CUDA(cudaEventRecord(e1, s));
-            g->pass_kernel = "fw_cluster_kernel";
-            g->pass_bytes = 12 * g->m + 8 * (int64_t)nact;
+            g->pass_kernel = "fw_resident_kernel";
+            g->pass_bytes = 8 * g->m + 8 * (int64_t)nact;
         } else if (fast) {
             LDS_CUDA(cudaEventRecord(e1, s));
             const std::string pk(g->pass_kernel);

@@ -14,8 +14,6 @@
 // in each handle is identical to what lds_fw would leave: W and R = D_N r as
 // exact integers, r in binary64.  Graphs that do not fit run the single-graph
 // path.
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <chrono>
 #include <map>
@@ -62,99 +60,6 @@ struct GraphJob {
     int64_t* R;         // [n] out: exact loads
     double* r;          // [n] out: reported loads
 };
-
-// ---- one mid-size graph on a thread-block cluster.  Every CTA of the cluster
-// keeps all load words in its shared memory and takes 1/CL_SIZE of the edges;
-// each counts its edges' receipts in its own shared memory.  After the pass,
-// CTA c owns the vertex slice c: it sums the slice's counts over the cluster's
-// shared memories (distributed shared memory), computes the new loads and
-// writes them into every CTA's copy.  Three cluster barriers per iteration
-// (after the pass, after the reads of the counts, after the broadcast) replace
-// grid-wide barriers.  Same iterates, ties and rounding as lds_fw.
-constexpr int CL_SIZE = 8;
-constexpr int CL_THREADS = 1024;
-constexpr int CL_SLICE = 4;       // vertices of the slice per thread (24,576 / 8 / 1,024 = 3)
-// 8 SMs against 152: past this many edges the grid-wide cooperative form wins
-// (measured at 500 iterations: 2.5 against 3.3 ms at 32k edges, 4.4 against
-// 4.3 ms at 64k, 12.7 against 5.1 ms at 348k)
-constexpr int64_t kClusterMaxEdges = 49152;
-
-template <bool FP32>
-__global__ void __launch_bounds__(CL_THREADS, 1) fw_cluster_kernel(GraphJob g, int32_t N, uint8_t* last) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    extern __shared__ __align__(16) uint32_t sm[];
-    const int32_t nv = g.nact;
-    uint32_t* L = sm;          // load words: R, or the bits of r in binary32
-    uint32_t* C = sm + nv;     // this CTA's counts
-    const unsigned rank = cl.block_rank(), cs = cl.num_blocks();
-    const int tid = threadIdx.x, bd = blockDim.x;
-    const int64_t e0 = g.m * rank / cs, e1 = g.m * (rank + 1) / cs;
-    const int32_t v0 = (int32_t)((int64_t)nv * rank / cs), v1 = (int32_t)((int64_t)nv * (rank + 1) / cs);
-    for (int32_t x = tid; x < nv; x += bd) {
-        const uint32_t d = (uint32_t)(g.rowptr[x + 1] - g.rowptr[x]);
-        L[x] = FP32 ? __float_as_uint(__fmul_rn((float)d, 0.5f)) : d;     // r0 = deg / 2, R0 = D_0 r0 = deg
-        C[x] = 0;
-    }
-    for (int64_t e = e0 + tid; e < e1; e += bd) g.wt[e] = 1u;             // W0 = D_0 / 2
-    cl.sync();
-    for (int32_t i = 1; i <= N; ++i) {
-        const uint32_t inc = 2u * (uint32_t)(i + 1);
-        for (int64_t e = e0 + tid; e < e1; e += bd) {
-            const int32_t u = g.eu[e], v = g.ev[e];
-            const uint32_t lu = L[u], lv = L[v];
-            const bool to_u = FP32 ? (__uint_as_float(lu) < __uint_as_float(lv)) : (lu < lv);
-            atomicAdd(C + (to_u ? u : v), 1u);
-            if (to_u) g.wt[e] += inc;
-            if (last && i == N) last[e] = to_u ? 1 : 0;
-        }
-        cl.sync();
-        uint32_t nl[CL_SLICE];
-        {
-            int j = 0;
-            for (int32_t x = v0 + tid; x < v1; x += bd, ++j) {
-                uint32_t c = 0;
-                for (unsigned r = 0; r < cs; ++r) c += cl.map_shared_rank(C, r)[x];
-                if (FP32) {
-                    const float gam = __fdiv_rn(2.0f, (float)(i + 2));
-                    const float om = __fsub_rn(1.0f, gam);
-                    nl[j] = __float_as_uint(__fadd_rn(__fmul_rn(om, __uint_as_float(L[x])), __fmul_rn(gam, (float)c)));
-                } else {
-                    nl[j] = L[x] + inc * c;
-                }
-            }
-        }
-        cl.sync();                               // every CTA has read the counts of its slice
-        for (int32_t x = tid; x < nv; x += bd) C[x] = 0;
-        {
-            int j = 0;
-            for (int32_t x = v0 + tid; x < v1; x += bd, ++j)
-                for (unsigned r = 0; r < cs; ++r) cl.map_shared_rank(L, r)[x] = nl[j];
-        }
-        cl.sync();
-    }
-    // outputs: W, R = the incident shares of W (D_N - W for the upper endpoint), r
-    const uint32_t D = (uint32_t)(N + 1) * (uint32_t)(N + 2);
-    for (int64_t e = e0 + tid; e < e1; e += bd) {
-        const uint32_t w = g.wt[e];
-        g.W[e] = (int64_t)w;
-        atomicAdd(C + g.eu[e], w);
-        atomicAdd(C + g.ev[e], D - w);
-    }
-    cl.sync();
-    for (int32_t x = v0 + tid; x < v1; x += bd) {
-        uint32_t c = 0;
-        for (unsigned r = 0; r < cs; ++r) c += cl.map_shared_rank(C, r)[x];
-        g.R[x] = (int64_t)c;
-        g.r[x] = FP32 ? (double)__uint_as_float(L[x]) : (double)L[x] / (double)D;
-    }
-    if (rank == 0)
-        for (int32_t x = nv + tid; x < g.n; x += bd) {
-            g.R[x] = 0;
-            g.r[x] = 0.0;
-        }
-    cl.sync();                                   // no CTA leaves while others read its counts
-}
 
 template <bool FP32>
 __global__ void __launch_bounds__(FB_THREADS)
@@ -248,49 +153,7 @@ void launch_bucket(const GraphJob* jobs, int32_t njobs, int32_t* next, int32_t m
     else LDS_LAUNCH(fw_batch_kernel<false>, grid, threads, smem, s, jobs, njobs, next, iters);
 }
 
-bool fits_on_chip(const lds_graph* g, int32_t N, lds_precision p);
-
 }  // namespace
-
-// Runs lds_fw's edge-density iterations of g on one cluster when its active
-// vertices fit in shared memory (exact or binary32); fills the handle's R, r, W
-// and, when `last` is given, the last iteration's choices.  False when the graph
-// does not fit or no cluster of CL_SIZE CTAs can be resident.
-bool fw_cluster_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last, bool any_size) {
-    static_assert(ONCHIP_MAX_V / CL_SIZE <= CL_SLICE * CL_THREADS, "a CTA's vertex slice exceeds its registers");
-    if (!fits_on_chip(g, N, p) || (!any_size && g->m > kClusterMaxEdges)) return false;
-    cudaStream_t s = g->stream;
-    const bool fp32 = p == LDS_FP32;
-    const size_t smem = (size_t)std::max(g->nact, 1) * 8;
-    const void* fn = fp32 ? (const void*)fw_cluster_kernel<true> : (const void*)fw_cluster_kernel<false>;
-    LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnchipSmemMax));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL_SIZE);
-    cfg.blockDim = dim3(CL_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CL_SIZE;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
-        cudaGetLastError();
-        return false;
-    }
-    DevBuf<uint32_t> wt(std::max<int64_t>(g->m, 1), s);
-    g->fw_W.alloc(std::max<int64_t>(g->m, 1), s);
-    GraphJob job{g->eu.get(), g->ev.get(), g->rowptr.get(), g->m, g->nact, g->n, wt.get(), g->fw_W.get(),
-                 g->fw_R.get(), g->fw_r.get()};
-    int32_t iters = N;
-    void* args[] = {(void*)&job, (void*)&iters, (void*)&last};
-    LDS_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return true;
-}
 
 namespace {
 
