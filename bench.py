@@ -53,7 +53,7 @@ PASS_TRAFFIC = {
 }
 PASS_SOURCE = {"fw_opass32_kernel": "paper_2504_10937_gb300/csrc/fw_oriented.cu",
                "fw_coop32_kernel": "paper_2504_10937_gb300/csrc/fw_oriented.cu",
-               "fw_tri_pass_kernel": "paper_2504_10937_gb300/csrc/fw.cu"}
+               "fw_tri_quad_kernel": "paper_2504_10937_gb300/csrc/fw_tri.cu"}
 GOLDEN = os.path.join(ROOT, "tests", "golden")
 
 
@@ -458,7 +458,7 @@ def run_ours(args):
     units = m_holder["units"]
     per_unit = ({"exact": 28, "fp32": 28, "fp64": 44} if tri else {"exact": 16, "fp32": 16, "fp64": 24})[args.precision]
     bytes_per_pass = per_unit * units
-    fused = pass_timing["pass_kernel"] == "fw_coop32_kernel"
+    fused = pass_timing["pass_kernel"] in ("fw_coop32_kernel", "fw_resident_kernel", "fw_tri_quad_kernel")
     if fused:
         # the cooperative kernel runs whole iterations: the pass and the vertex
         # update (16 B per vertex), timed per launch and divided by the iterations

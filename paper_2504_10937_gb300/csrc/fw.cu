@@ -17,10 +17,6 @@
 // planes are folded into per-slot weights W = D_N alpha every K iterations:
 // W_slot += sum_i 2(i+1) bit_i.
 //
-// Triangle pass: one thread per triangle (a < b < c): the receiving vertex is
-// the lowest-load one, ties to the larger id (later column); the column is
-// stored as two bit planes and the count is added with warp-aggregated atomics.
-//
 // The binary64 path is Alg. 1 literally: one alpha per slot updated as
 // alpha = (1 - gamma) alpha + gamma alpha_hat, then r_x summed over row x left
 // to right by one thread per row.
@@ -247,105 +243,6 @@ __global__ void pad_i64_kernel(int64_t* p, int32_t from, int32_t to) {
 
 // ---- triangles
 
-template <class L>
-__global__ void __launch_bounds__(FW_THREADS) fw_tri_pass_kernel(const int32_t* __restrict__ ta,
-                                                                 const int32_t* __restrict__ tb,
-                                                                 const int32_t* __restrict__ tc, int64_t ntri,
-                                                                 const L* __restrict__ R, int32_t* __restrict__ cnt,
-                                                                 uint32_t* __restrict__ plane0,
-                                                                 uint32_t* __restrict__ plane1) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t nchunks = (ntri + 31) >> 5;
-    for (int64_t g0 = warp * FW_UNROLL; g0 < nchunks; g0 += nwarps * FW_UNROLL) {
-        int32_t a[FW_UNROLL], b[FW_UNROLL], c[FW_UNROLL];
-#pragma unroll
-        for (int k = 0; k < FW_UNROLL; ++k) {
-            int64_t t = ((g0 + k) << 5) + lane;
-            bool ok = t < ntri;
-            a[k] = ok ? __ldg(ta + t) : 0;
-            b[k] = ok ? __ldg(tb + t) : 0;
-            c[k] = ok ? __ldg(tc + t) : 0;
-        }
-        L ra[FW_UNROLL], rb[FW_UNROLL], rc[FW_UNROLL];
-#pragma unroll
-        for (int k = 0; k < FW_UNROLL; ++k) {
-            int64_t t = ((g0 + k) << 5) + lane;
-            if (t < ntri) {
-                ra[k] = __ldg(R + a[k]);
-                rb[k] = __ldg(R + b[k]);
-                rc[k] = __ldg(R + c[k]);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < FW_UNROLL; ++k) {
-            int64_t g = g0 + k;
-            int64_t t = (g << 5) + lane;
-            bool ok = t < ntri;
-            int best = 2;
-            int32_t w = c[k];
-            if (ok) {
-                L bv = rc[k];
-                if (rb[k] < bv) { best = 1; bv = rb[k]; w = b[k]; }
-                if (ra[k] < bv) { best = 0; w = a[k]; }
-            }
-            uint32_t b0 = __ballot_sync(FULL, ok && (best & 1));
-            uint32_t b1 = __ballot_sync(FULL, ok && (best & 2));
-            if (g < nchunks && lane == 0) {
-                plane0[g] = b0;
-                plane1[g] = b1;
-            }
-            uint32_t okmask = __ballot_sync(FULL, ok);
-            if (ok) {
-                uint32_t peers = __match_any_sync(okmask, w);
-                if ((peers & ((1u << lane) - 1u)) == 0) atomicAdd(cnt + w, __popc(peers));
-            }
-        }
-    }
-}
-
-// Wt[3t + k] += sum_planes [column == k] * (mult * (i_first + j + 1))
-__global__ void fw_tri_fold_kernel(const uint32_t* __restrict__ planes, int nplanes, int64_t nchunks, int64_t ntri,
-                                   int64_t i_first, int64_t mult, uint32_t* __restrict__ Wt) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntri; t += stride) {
-        int64_t g = t >> 5;
-        int lane = (int)(t & 31);
-        uint32_t acc[3] = {0, 0, 0};
-        for (int j = 0; j < nplanes; ++j) {
-            uint32_t p0 = (__ldg(planes + (2 * (int64_t)j) * nchunks + g) >> lane) & 1u;
-            uint32_t p1 = (__ldg(planes + (2 * (int64_t)j + 1) * nchunks + g) >> lane) & 1u;
-            uint32_t col = p0 | (p1 << 1);
-            uint32_t inc = (uint32_t)(mult * (i_first + j + 1));
-            acc[0] += col == 0 ? inc : 0u;
-            acc[1] += col == 1 ? inc : 0u;
-            acc[2] += col == 2 ? inc : 0u;
-        }
-        Wt[3 * t] += acc[0];
-        Wt[3 * t + 1] += acc[1];
-        Wt[3 * t + 2] += acc[2];
-    }
-}
-
-__global__ void tri_counts_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t ntri, int32_t* tcount) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntri; t += stride) {
-        atomicAdd(tcount + ta[t], 1);
-        atomicAdd(tcount + tb[t], 1);
-        atomicAdd(tcount + tc[t], 1);
-    }
-}
-
-__global__ void init_loads_tri_kernel(const int32_t* tcount, int32_t nact, int64_t* R, float* r32) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride) {
-        int32_t t = tcount[x];
-        if (R) R[x] = 2 * (int64_t)t;
-        if (r32) r32[x] = __fdiv_rn((float)t, 3.0f);
-    }
-}
-
 __global__ void tri_loads_from_w_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t ntri,
                                         const uint32_t* Wt, unsigned long long* R) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -353,14 +250,6 @@ __global__ void tri_loads_from_w_kernel(const int32_t* ta, const int32_t* tb, co
         atomicAdd(R + ta[t], (unsigned long long)Wt[3 * t]);
         atomicAdd(R + tb[t], (unsigned long long)Wt[3 * t + 1]);
         atomicAdd(R + tc[t], (unsigned long long)Wt[3 * t + 2]);
-    }
-}
-
-__global__ void tri_last_kernel(const uint32_t* plane0, const uint32_t* plane1, int64_t ntri, uint8_t* last) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntri; t += stride) {
-        uint32_t p0 = (plane0[t >> 5] >> (t & 31)) & 1u, p1 = (plane1[t >> 5] >> (t & 31)) & 1u;
-        last[t] = (uint8_t)(p0 | (p1 << 1));
     }
 }
 
@@ -537,13 +426,9 @@ __global__ void tri_w_from_alpha64_kernel(const double* alpha, int64_t ntri, int
 }
 
 struct TriFwState {
-    DevBuf<int64_t> R;
-    DevBuf<float> r32;
-    DevBuf<double> r64;        // binary64 form
-    DevBuf<uint8_t> last64;    // binary64 form: receiving column of the last iteration
+    DevBuf<double> r64;
+    DevBuf<uint8_t> last64;    // receiving column of the last iteration
     DevBuf<uint32_t> W;        // [3 ntri]
-    DevBuf<uint32_t> planes;   // 2 planes per stored iteration
-    int64_t last_pair = -1;
 };
 
 static void run_tri_fw64(lds_graph* g, int N, TriFwState& st, PassTimer& timer) {
@@ -573,71 +458,6 @@ static void run_tri_fw64(lds_graph* g, int N, TriFwState& st, PassTimer& timer) 
     }
     const int64_t Dn3 = 3 * (int64_t)(N + 1) * (N + 2);
     if (ntri) LDS_LAUNCH(tri_w_from_alpha64_kernel, grid_for(ntri, blk), blk, 0, s, alpha.get(), ntri, Dn3, st.W.get());
-}
-
-static void run_tri_fw(lds_graph* g, int N, lds_precision p, TriFwState& st, PassTimer& timer) {
-    cudaStream_t s = g->stream;
-    const int64_t ntri = g->ntri;
-    const int64_t nchunks = (ntri + 31) / 32;
-    const int32_t nact = g->nact;
-    const int blk = 256;
-    DevBuf<int32_t> cnt(std::max<int32_t>(nact, 1), s);
-    LDS_CUDA(cudaMemsetAsync(cnt.get(), 0, std::max<int32_t>(nact, 1) * sizeof(int32_t), s));
-    DevBuf<int32_t> tcount(std::max<int32_t>(nact, 1), s);
-    LDS_CUDA(cudaMemsetAsync(tcount.get(), 0, std::max<int32_t>(nact, 1) * sizeof(int32_t), s));
-    if (ntri) LDS_LAUNCH(tri_counts_kernel, grid_for(ntri, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), ntri, tcount.get());
-    LDS_CHECK_LAUNCH();
-    const int K = planes_capacity(2 * nchunks, N);
-    st.planes.alloc(std::max<int64_t>(1, 2 * (int64_t)K * nchunks), s);
-    st.W.alloc(std::max<int64_t>(3 * ntri, 1), s);
-    if (ntri) LDS_LAUNCH(fill_u32_kernel, grid_for(3 * ntri, blk), blk, 0, s, st.W.get(), 3 * ntri, 2u);
-    if (p == LDS_EXACT) {
-        st.R.alloc(std::max<int32_t>(nact, 1), s);
-        if (nact) LDS_LAUNCH(init_loads_tri_kernel, grid_for(nact, blk), blk, 0, s, tcount.get(), nact, st.R.get(), nullptr);
-    } else {
-        st.r32.alloc(std::max<int32_t>(nact, 1), s);
-        if (nact) LDS_LAUNCH(init_loads_tri_kernel, grid_for(nact, blk), blk, 0, s, tcount.get(), nact, nullptr, st.r32.get());
-    }
-    LDS_CHECK_LAUNCH();
-    const int grid = fw_grid(nchunks);
-    int stored = 0;
-    int64_t first_i = 1;
-    for (int i = 1; i <= N; ++i) {
-        uint32_t* p0 = st.planes.get() + (2 * (int64_t)stored) * nchunks;
-        uint32_t* p1 = p0 + nchunks;
-        if (nchunks) {
-            timer.start(s);
-            if (p == LDS_EXACT)
-                LDS_LAUNCH(fw_tri_pass_kernel<int64_t>, grid, FW_THREADS, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), ntri,
-                                                                       st.R.get(), cnt.get(), p0, p1);
-            else
-                LDS_LAUNCH(fw_tri_pass_kernel<float>, grid, FW_THREADS, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), ntri,
-                                                                     st.r32.get(), cnt.get(), p0, p1);
-            timer.stop(s);
-            LDS_CHECK_LAUNCH();
-            if (p == LDS_EXACT) {
-                LDS_LAUNCH(fw_update_exact_kernel, grid_for(nact, blk), blk, 0, s, st.R.get(), cnt.get(), nact, 6 * (int64_t)(i + 1));
-            } else {
-                float gam = 2.0f / (float)(i + 2);
-                float om = 1.0f - gam;
-                LDS_LAUNCH(fw_update_fp32_kernel, grid_for(nact, blk), blk, 0, s, st.r32.get(), cnt.get(), nact, gam, om);
-            }
-            LDS_CHECK_LAUNCH();
-        }
-        ++stored;
-        if (stored == K || i == N) {
-            if (ntri) {
-                LDS_LAUNCH(fw_tri_fold_kernel, grid_for(ntri, blk), blk, 0, s, st.planes.get(), stored, nchunks, ntri, first_i, 6,
-                                                                      st.W.get());
-                LDS_CHECK_LAUNCH();
-            }
-            st.last_pair = stored - 1;
-            if (i < N) {
-                stored = 0;
-                first_i = i + 1;
-            }
-        }
-    }
 }
 
 void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool want_last) {
@@ -721,42 +541,33 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
         }
     } else {
         ensure_triangles(g);
-        TriFwState st;
+        const int64_t ntri = g->ntri;
         LDS_CUDA(cudaEventRecord(e0, s));
-        if (p == LDS_FP64) run_tri_fw64(g, iters, st, timer);
-        else run_tri_fw(g, iters, p, st, timer);
-        LDS_CUDA(cudaEventRecord(e1, s));
-        if (p == LDS_FP64) {
+        if (p != LDS_FP64) {
+            run_tri_fw(g, iters, p, want_last, timer);
+            LDS_CUDA(cudaEventRecord(e1, s));
+            g->pass_kernel = "fw_tri_quad_kernel";
+            // c, two choice bits and a group's (a, b) per quad of triangles; loads read and
+            // written and receipts per vertex
+            g->pass_bytes = 17 * g->tv_nq + 8 * ((g->tv_nq + 31) / 32) + (p == LDS_EXACT ? 24 : 16) * (int64_t)nact;
+        } else {
+            TriFwState st;
+            run_tri_fw64(g, iters, st, timer);
+            LDS_CUDA(cudaEventRecord(e1, s));
             g->pass_kernel = "tri_pass64_kernel";
             g->pass_bytes = 12 * g->ntri + 48 * g->ntri + 24 * (int64_t)nact;
-        } else {
-            g->pass_kernel = "fw_tri_pass_kernel";
-            g->pass_bytes = 12 * g->ntri + 8 * ((g->ntri + 31) / 32) + (p == LDS_EXACT ? 8 : 4) * (int64_t)nact;
-        }
-        const int64_t ntri = g->ntri;
-        LDS_CUDA(cudaMemsetAsync(R_int.get(), 0, std::max(n, 1) * sizeof(int64_t), s));
-        if (ntri)
-            LDS_LAUNCH(tri_loads_from_w_kernel, grid_for(ntri, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), ntri,
-                       st.W.get(), (unsigned long long*)R_int.get());
-        if (n) {
-            if (p == LDS_EXACT)
-                LDS_LAUNCH(loads_to_double_kernel<int64_t>, grid_for(n, blk), blk, 0, s, st.R.get(), nact, n, (double)Dn, r_int.get());
-            else if (p == LDS_FP64)
+            LDS_CUDA(cudaMemsetAsync(R_int.get(), 0, std::max(n, 1) * sizeof(int64_t), s));
+            if (ntri)
+                LDS_LAUNCH(tri_loads_from_w_kernel, grid_for(ntri, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(),
+                           ntri, st.W.get(), (unsigned long long*)R_int.get());
+            if (n)
                 LDS_LAUNCH(loads_to_double_kernel<double>, grid_for(n, blk), blk, 0, s, st.r64.get(), nact, n, 1.0, r_int.get());
-            else
-                LDS_LAUNCH(loads_to_double_kernel<float>, grid_for(n, blk), blk, 0, s, st.r32.get(), nact, n, 1.0, r_int.get());
-        }
-        g->fw_W.alloc(std::max<int64_t>(3 * ntri, 1), s);
-        if (ntri) LDS_LAUNCH(widen_u32_kernel, grid_for(3 * ntri, blk), blk, 0, s, st.W.get(), 3 * ntri, g->fw_W.get());
-        if (want_last) {
-            g->fw_last.alloc(std::max<int64_t>(ntri, 1), s);
-            int64_t nch = (ntri + 31) / 32;
-            const uint32_t* p0 = st.planes.get() + 2 * std::max<int64_t>(st.last_pair, 0) * nch;
-            if (ntri) {
-                if (p == LDS_FP64)
+            g->fw_W.alloc(std::max<int64_t>(3 * ntri, 1), s);
+            if (ntri) LDS_LAUNCH(widen_u32_kernel, grid_for(3 * ntri, blk), blk, 0, s, st.W.get(), 3 * ntri, g->fw_W.get());
+            if (want_last) {
+                g->fw_last.alloc(std::max<int64_t>(ntri, 1), s);
+                if (ntri)
                     LDS_CUDA(cudaMemcpyAsync(g->fw_last.get(), st.last64.get(), ntri, cudaMemcpyDeviceToDevice, s));
-                else if (iters == 0) LDS_CUDA(cudaMemsetAsync(g->fw_last.get(), 2, ntri, s));
-                else LDS_LAUNCH(tri_last_kernel, grid_for(ntri, blk), blk, 0, s, p0, p0 + nch, ntri, g->fw_last.get());
             }
         }
     }

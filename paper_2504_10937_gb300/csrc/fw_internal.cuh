@@ -73,4 +73,7 @@ struct EdgeFwOut {
 bool run_edge_fw_oriented(lds_graph* g, int N, lds_precision p, bool want_w, bool want_last, EdgeFwOut& out,
                           PassTimer& timer);
 
+// Triangle FW (Alg. 6), exact and binary32: fills g->fw_R, fw_r, fw_W (and fw_last).
+void run_tri_fw(lds_graph* g, int N, lds_precision p, bool want_last, PassTimer& timer);
+
 }  // namespace lds

@@ -346,9 +346,12 @@ void set_stream(lds_graph* g, cudaStream_t s) {
     g->fwv_chunk_nz0.s = s;
     g->fwv_edge.s = s;
     g->fwv_rowptr.s = s;
-    g->fwv_ta.s = s;
-    g->fwv_tb.s = s;
-    g->fwv_tc.s = s;
+    g->tv_perm.s = s;
+    g->tv_count.s = s;
+    g->tv_c.s = s;
+    g->tv_qt.s = s;
+    g->tv_chunk_g0.s = s;
+    g->tv_grp.s = s;
     g->fw_R.s = s;
     g->fw_r.s = s;
     g->fw_W.s = s;

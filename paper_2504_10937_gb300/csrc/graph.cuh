@@ -49,7 +49,16 @@ struct lds_graph {
     lds::DevBuf<int32_t> fwv_chunk_nz0;// [ceil(m / 32)] non-empty-row index of slot 32 g
     lds::DevBuf<int64_t> fwv_edge;     // [m] canonical edge id of each slot
     lds::DevBuf<int32_t> fwv_rowptr;   // [nact + 1] slots of the row of fw id p: rowptr[p] .. rowptr[p+1]
-    lds::DevBuf<int32_t> fwv_ta, fwv_tb, fwv_tc;  // triangles in fw ids (lazy)
+
+    // triangle FW view (lazy, fw_tri.cu): vertices ranked by (triangle count descending,
+    // id ascending); the triangles of one (a, b) consecutive, c in quads
+    int64_t tv_nq = 0;
+    lds::DevBuf<int32_t> tv_perm;      // [nact] rank -> internal id
+    lds::DevBuf<uint32_t> tv_count;    // [nact] triangles of the vertex of each rank
+    lds::DevBuf<int32_t> tv_c;         // [4 tv_nq, padded to chunks] rank of c; bit 31: first quad of a group
+    lds::DevBuf<uint32_t> tv_qt;       // [tv_nq] triangle of each quad's first entry
+    lds::DevBuf<int32_t> tv_chunk_g0;  // group of the first quad of each 32-quad chunk
+    lds::DevBuf<int2> tv_grp;          // (a, b) of each group, as ranks
 
     // state of the most recent Frank-Wolfe run (internal ids), read by the later stages
     bool fw_valid = false;
