@@ -47,12 +47,9 @@ UNIT_TRI = "triangle-updates/s"
 # from at capture time.  A kernel whose source changed since has no matching entry
 # and reports null.
 PASS_TRAFFIC = {
-    # one 20-iteration launch on the 1M-vertex workload (64,239,872 B read + 4,828,928 B
-    # written, the cold first read of the view included), per iteration
-    ("fw_coop32_kernel", "exact", "1df8d6eea5f0f836"): 3453440,
 }
 PASS_SOURCE = {"fw_opass32_kernel": "paper_2504_10937_gb300/csrc/fw_oriented.cu",
-               "fw_coop32_kernel": "paper_2504_10937_gb300/csrc/fw_oriented.cu",
+               "fw_quad_kernel": "paper_2504_10937_gb300/csrc/fw_quads.cu",
                "fw_tri_quad_kernel": "paper_2504_10937_gb300/csrc/fw_tri.cu"}
 GOLDEN = os.path.join(ROOT, "tests", "golden")
 
@@ -458,7 +455,7 @@ def run_ours(args):
     units = m_holder["units"]
     per_unit = ({"exact": 28, "fp32": 28, "fp64": 44} if tri else {"exact": 16, "fp32": 16, "fp64": 24})[args.precision]
     bytes_per_pass = per_unit * units
-    fused = pass_timing["pass_kernel"] in ("fw_coop32_kernel", "fw_resident_kernel", "fw_tri_quad_kernel")
+    fused = pass_timing["pass_kernel"] in ("fw_quad_kernel", "fw_resident_kernel", "fw_tri_quad_kernel")
     if fused:
         # the cooperative kernel runs whole iterations: the pass and the vertex
         # update (16 B per vertex), timed per launch and divided by the iterations

@@ -388,21 +388,21 @@ int32_t lds_debug_pick_next(int32_t nq, const int64_t* bytes, const uint8_t* gra
  *      and exact load below 2^32) runs with its slots resident, each endpoint
  *      deciding its own edges, one barrier per iteration over one CTA, a
  *      cluster of 8 or up to one CTA per SM; otherwise the degree-oriented
- *      pass (each edge once, stored at its
- *      lower-degree endpoint, hot loads in shared memory) with 32-bit load
- *      words when every scaled load fits 32 bits, else with 64-bit keys
- *      (load, id), else variant 1.  With 32-bit words the pass counts only
- *      the receipts of the stored targets; the vertex update adds each row
- *      endpoint's receipts as the popcount of its row's bits in the
- *      iteration's choice plane, and many iterations (pass, grid barrier,
- *      update, grid barrier) run in one cooperative launch;
+ *      pass with 32-bit load words, when every degree is below 65,536 and
+ *      every scaled load below 2^32 (each edge once, stored at its
+ *      lower-degree endpoint, four targets to a lane, hot loads in shared
+ *      memory; the pass counts the receipts of the stored targets, the vertex
+ *      update adds each row endpoint's as the popcount of its row's bits in
+ *      the iteration's choice plane; many iterations - pass, grid barrier,
+ *      update, grid barrier - run in one cooperative launch); else the same
+ *      orientation with 64-bit keys (load, id), else variant 1;
  *   1  the symmetric-CSR pass (each edge twice, once from each endpoint);
  *   2  the degree-oriented pass with 64-bit keys;
- *   3  as 0 with 32-bit words, both endpoints' receipts counted inside the
- *      pass, one pass launch and one update launch per iteration;
- *   4  as 0 with 32-bit words, one pass launch and one update launch per
- *      iteration;
- *   5  as 0 without the resident form (the cooperative launch for every size);
+ *   3  the degree-oriented pass with 32-bit words, one slot a lane, both
+ *      endpoints' receipts counted inside the pass, one pass launch and one
+ *      update launch per iteration;
+ *   4  as 3 with the row endpoints' receipts counted by the update;
+ *   5  as 0 without the resident form (the cooperative pass for every size);
  *   6  as 0 (kept for callers of the former cluster form).
  * All compute the same iterates.  Errors: LDS_EINVAL. */
 lds_status lds_set_fw_variant(int32_t variant);

@@ -491,19 +491,23 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
             if (res) timer.stop(s, iters);
             else g->fw_last.release();
         }
-        bool fast = !res && g_fw_variant != 1 && run_edge_fw_oriented(g, iters, p, true, want_last, fo, timer);
+        const bool quads = !res && (g_fw_variant == 0 || g_fw_variant == 5 || g_fw_variant == 6) &&
+                           run_edge_fw_quads(g, iters, p, want_last, timer);
+        bool fast = !res && !quads && g_fw_variant != 1 && run_edge_fw_oriented(g, iters, p, true, want_last, fo, timer);
         if (res) {
             LDS_CUDA(cudaEventRecord(e1, s));
             g->pass_kernel = "fw_resident_kernel";
             g->pass_bytes = 8 * g->m + 8 * (int64_t)nact;
+        } else if (quads) {
+            LDS_CUDA(cudaEventRecord(e1, s));
+            g->pass_kernel = "fw_quad_kernel";
+            // four targets, the row and four choice bits (written, read again) per quad; loads
+            // read and written, counts and row ranges per vertex
+            g->pass_bytes = 21 * g->fwq_nq + 24 * (int64_t)nact;
         } else if (fast) {
             LDS_CUDA(cudaEventRecord(e1, s));
             const std::string pk(g->pass_kernel);
-            g->pass_bytes = 4 * g->m + 8 * ((g->m + 31) / 32) + 4 * g->fwv_nz +
-                            (pk == "fw_opass32_kernel" || pk == "fw_coop32_kernel" ? 4 : 8) * (int64_t)nact;
-            // the cooperative kernel also runs the vertex update: words and counts read and
-            // written, row ranges read, the plane read again
-            if (pk == "fw_coop32_kernel") g->pass_bytes += 20 * (int64_t)nact + 4 * ((g->m + 31) / 32);
+            g->pass_bytes = 4 * g->m + 8 * ((g->m + 31) / 32) + 4 * g->fwv_nz + (pk == "fw_opass32_kernel" ? 4 : 8) * (int64_t)nact;
             R_int = std::move(fo.R_int);
             r_int = std::move(fo.r_int);
             g->fw_W = std::move(fo.W_edge);
@@ -547,9 +551,9 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
             run_tri_fw(g, iters, p, want_last, timer);
             LDS_CUDA(cudaEventRecord(e1, s));
             g->pass_kernel = "fw_tri_quad_kernel";
-            // c, two choice bits and a group's (a, b) per quad of triangles; loads read and
-            // written and receipts per vertex
-            g->pass_bytes = 17 * g->tv_nq + 8 * ((g->tv_nq + 31) / 32) + (p == LDS_EXACT ? 24 : 16) * (int64_t)nact;
+            // c and two choice bits per entry, (a, b) per group; loads read and written and
+            // receipts per vertex
+            g->pass_bytes = 548 * g->tv_chunks + 8 * (int64_t)g->tv_grp.n + (p == LDS_EXACT ? 24 : 16) * (int64_t)nact;
         } else {
             TriFwState st;
             run_tri_fw64(g, iters, st, timer);

@@ -73,6 +73,16 @@ struct EdgeFwOut {
 bool run_edge_fw_oriented(lds_graph* g, int N, lds_precision p, bool want_w, bool want_last, EdgeFwOut& out,
                           PassTimer& timer);
 
+// Folds the choice planes of quad layouts (word j, bit l of a chunk is entry 4 l + j)
+// into weights: W[entry] += mult * (i_first + k + 1) per set bit of plane k.  With W1
+// the planes come in pairs, the second of each pair for W1.
+void fold_quads(const uint32_t* planes, int nplanes, int64_t nchunks, int64_t i_first, uint32_t mult, uint32_t* W0,
+                uint32_t* W1, cudaStream_t s);
+
+// Edge FW over quads of targets (fw_quads.cu): fills g->fw_R, fw_r, fw_W (and fw_last).
+// False when the scaled loads or a degree do not fit its words.
+bool run_edge_fw_quads(lds_graph* g, int N, lds_precision p, bool want_last, PassTimer& timer);
+
 // Triangle FW (Alg. 6), exact and binary32: fills g->fw_R, fw_r, fw_W (and fw_last).
 void run_tri_fw(lds_graph* g, int N, lds_precision p, bool want_last, PassTimer& timer);
 

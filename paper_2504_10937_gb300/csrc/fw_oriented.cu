@@ -18,10 +18,7 @@
 // count is the popcount of its lanes (one atomic per row segment); the
 // target's count goes to shared memory for hot targets (flushed once per
 // block) and to a global atomic otherwise.
-#include <cooperative_groups.h>
-
 #include <algorithm>
-#include <type_traits>
 
 #include "fw_internal.cuh"
 #include "prims.cuh"
@@ -222,32 +219,23 @@ __global__ void __launch_bounds__(OP_THREADS, 1)
 // 16-bit counters packed two per word.  Ties (equal words) are rare and are
 // broken by the internal ids, looked up only then.
 constexpr int HOT32 = 32768;
-// cooperative FW: hot vertices' global counts packed two per word (one atomic per
-// word in the flush), and the grid sized to the work (chunks per block; 0: one
-// block per SM whatever the size).  Both measured slower on the 1M-vertex graph
-// and its refinement subgraphs, so both are off.
-constexpr bool kPackedHot = false;
-constexpr int kCoopChunksPerBlock = 0;
 constexpr size_t OP32_SMEM = (size_t)HOT32 * 4 + (size_t)HOT32 * 2;
 
 // One pass over every stored slot.  ROWS: the row endpoints' counts are left
 // out of the pass; the vertex update takes them as popcounts of each row's bit
-// range in this iteration's plane.  COOP: the body runs inside a cooperative
-// kernel whose other blocks rewrite the load words between passes, so words
-// are read through L2 (never the read-only data path).
-template <int U, class Word, bool ROWS, bool COOP>
+// range in this iteration's plane.
+template <int U, class Word, bool ROWS>
 __device__ __forceinline__ void opass32_body(const int32_t* __restrict__ col, const int32_t* __restrict__ chunk_nz0,
                                              const int32_t* __restrict__ nzrow, int64_t nslots, int64_t nchunks,
                                              const Word* word, const int32_t* __restrict__ perm, int32_t nhot,
-                                             int32_t* cnt, uint32_t* plane, Word* hword, uint32_t* hcnt2,
-                                             uint32_t* hglob = nullptr) {
+                                             int32_t* cnt, uint32_t* plane, Word* hword, uint32_t* hcnt2) {
     {
         const uint4* w4 = reinterpret_cast<const uint4*>(word);
         uint4* h4 = reinterpret_cast<uint4*>(hword);
         const int n4 = nhot >> 2;
 #pragma unroll 8
-        for (int i = threadIdx.x; i < n4; i += blockDim.x) h4[i] = COOP ? __ldcg(w4 + i) : __ldg(w4 + i);
-        for (int i = (n4 << 2) + threadIdx.x; i < nhot; i += blockDim.x) hword[i] = COOP ? __ldcg(word + i) : __ldg(word + i);
+        for (int i = threadIdx.x; i < n4; i += blockDim.x) h4[i] = __ldg(w4 + i);
+        for (int i = (n4 << 2) + threadIdx.x; i < nhot; i += blockDim.x) hword[i] = __ldg(word + i);
         uint4* c4 = reinterpret_cast<uint4*>(hcnt2);
         for (int i = threadIdx.x; i < (nhot + 7) >> 3; i += blockDim.x) c4[i] = make_uint4(0, 0, 0, 0);
     }
@@ -328,18 +316,10 @@ __device__ __forceinline__ void opass32_body(const int32_t* __restrict__ col, co
         }
     }
     __syncthreads();
-    // hglob: the hot vertices' global counts, packed like the shared ones (a vertex
-    // receives at most its degree < 2^16 per iteration, so halves never carry)
     for (int i = threadIdx.x; i < (nhot + 1) >> 1; i += blockDim.x) {
         uint32_t v = hcnt2[i];
-        if (v) {
-            if (hglob) {
-                atomicAdd(hglob + i, v);
-            } else {
-                if (v & 0xffffu) atomicAdd(cnt + 2 * i, (int)(v & 0xffffu));
-                if (v >> 16) atomicAdd(cnt + 2 * i + 1, (int)(v >> 16));
-            }
-        }
+        if (v & 0xffffu) atomicAdd(cnt + 2 * i, (int)(v & 0xffffu));
+        if (v >> 16) atomicAdd(cnt + 2 * i + 1, (int)(v >> 16));
     }
 }
 
@@ -352,7 +332,7 @@ __global__ void __launch_bounds__(OP_THREADS, 1)
     extern __shared__ __align__(16) unsigned char smem[];
     Word* hword = reinterpret_cast<Word*>(smem);
     uint32_t* hcnt2 = reinterpret_cast<uint32_t*>(smem + (size_t)HOT32 * 4);   // two 16-bit counters per word
-    opass32_body<U, Word, ROWS, false>(col, chunk_nz0, nzrow, nslots, nchunks, word, perm, nhot, cnt, plane, hword,
+    opass32_body<U, Word, ROWS>(col, chunk_nz0, nzrow, nslots, nchunks, word, perm, nhot, cnt, plane, hword,
                                        hcnt2);
 }
 
@@ -417,75 +397,6 @@ __global__ void oword_update_rows_fp32_kernel(float* __restrict__ r32, int32_t* 
         const int32_t c = t + row_receipts(rowptr, plane, p);
         r32[p] = __fadd_rn(__fmul_rn(one_minus, r32[p]), __fmul_rn(gam, (float)c));
         if (t) cnt[p] = 0;
-    }
-}
-
-// Iterations i_first .. i_first + K - 1 in one cooperative launch: each runs
-// the pass (targets' receipts; choice plane it of `planes`), a grid barrier,
-// the vertex update (row endpoints' receipts from the plane, then R += 2(i+1) c
-// for the exact words or r <- (1 - gamma) r + gamma c in binary32 with gamma =
-// fl(2 / (i + 2))), and a second barrier before the next pass stages the new
-// words.  Same iterates, ties and rounding as the per-iteration launches.
-template <class Word>
-__global__ void __launch_bounds__(OP_THREADS, 1)
-    fw_coop32_kernel(const int32_t* __restrict__ col, const int32_t* __restrict__ chunk_nz0,
-                     const int32_t* __restrict__ nzrow, int64_t nslots, int64_t nchunks, Word* word,
-                     const int32_t* __restrict__ perm, int32_t nhot, int32_t* cnt, const int32_t* __restrict__ rowptr,
-                     uint32_t* planes, int32_t nact, int32_t i_first, int32_t K, uint32_t* hglob) {
-    cooperative_groups::grid_group grid = cooperative_groups::this_grid();
-    extern __shared__ __align__(16) unsigned char smem[];
-    Word* hword = reinterpret_cast<Word*>(smem);
-    uint32_t* hcnt2 = reinterpret_cast<uint32_t*>(smem + (size_t)HOT32 * 4);
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    for (int32_t it = 0; it < K; ++it) {
-        const int32_t i = i_first + it;
-        uint32_t* plane = planes + (int64_t)it * nchunks;
-        opass32_body<OP_UNROLL, Word, true, true>(col, chunk_nz0, nzrow, nslots, nchunks, word, perm, nhot, cnt, plane,
-                                                  hword, hcnt2, kPackedHot ? hglob : nullptr);
-        grid.sync();
-        // update: one work item per packed word of hot counts (two vertices), then one
-        // per cold vertex; without packing, one item per vertex
-        const int32_t hw = kPackedHot ? (nhot + 1) >> 1 : 0;
-        const int64_t items = (int64_t)hw + (nact - (kPackedHot ? nhot : 0));
-        for (int64_t it = tid; it < items; it += nthreads) {
-            int32_t p0, np;
-            uint32_t packed = 0;
-            int32_t tc = 0;
-            if (it < hw) {
-                p0 = (int32_t)(2 * it);
-                np = min(2, nhot - p0);
-                packed = __ldcg(hglob + it);
-                if (packed) hglob[it] = 0;
-            } else {
-                p0 = (kPackedHot ? nhot : 0) + (int32_t)(it - hw);
-                np = 1;
-                tc = __ldcg(cnt + p0);
-                if (tc) cnt[p0] = 0;
-            }
-            for (int32_t j = 0; j < np; ++j) {
-                const int32_t p = p0 + j;
-                int32_t c = it < hw ? (int32_t)((packed >> (16 * j)) & 0xffffu) : tc;
-                const int32_t a = rowptr[p], b = rowptr[p + 1];
-                if (a < b) {
-                    const int32_t wa = a >> 5, wb = (b - 1) >> 5;
-                    for (int32_t q = wa; q <= wb; ++q) {
-                        uint32_t bits = __ldcg(plane + q);
-                        if (q == wa) bits &= FULL << (a & 31);
-                        if (q == wb) bits &= lanes_le((b - 1) & 31);
-                        c += __popc(bits);
-                    }
-                }
-                if constexpr (std::is_same<Word, float>::value) {
-                    const float gam = __fdiv_rn(2.0f, (float)(i + 2));
-                    const float om = __fsub_rn(1.0f, gam);
-                    word[p] = __fadd_rn(__fmul_rn(om, word[p]), __fmul_rn(gam, (float)c));
-                } else {
-                    if (c) word[p] += (uint32_t)(2 * (i + 1)) * (uint32_t)c;
-                }
-            }
-        }
-        grid.sync();
     }
 }
 
@@ -629,15 +540,14 @@ void fold_planes(const uint32_t* planes, int nplanes, int64_t nchunks, int64_t n
     LDS_LAUNCH(fold_tiled_kernel, grid, 1024, 0, s, planes, nplanes, nchunks, nitems, i_first, mult, W);
 }
 
-void ensure_fw_view(lds_graph* g) {
-    if (g->fwv_built) return;
+void ensure_fw_ranks(lds_graph* g) {
+    if (g->fwv_perm.p) return;
     cudaStream_t s = g->stream;
     const int32_t nact = g->nact;
-    const int64_t m = g->m;
     const int blk = 256;
     int bits = std::max(1, bit_length_u64((uint64_t)std::max(nact, 1)));
     g->fwv_bits = bits;
-    g->fwv_perm.alloc(std::max(nact, 1), s);
+    DevBuf<int32_t> perm(std::max(nact, 1), s);
     g->fwv_pos.alloc(std::max(nact, 1), s);
     if (nact > 0) {
         DevBuf<uint64_t> rk(nact, s);
@@ -645,9 +555,19 @@ void ensure_fw_view(lds_graph* g) {
         LDS_LAUNCH(rank_keys_kernel, grid_for(nact, blk), blk, 0, s, g->rowptr.get(), nact, maxdeg, bits, rk.get());
         radix_sort_u64(rk.get(), nullptr, nact, bits + bit_length_u64((uint64_t)maxdeg), s);
         uint64_t mask = (1ull << bits) - 1ull;
-        LDS_LAUNCH(perm_from_keys_kernel, grid_for(nact, blk), blk, 0, s, rk.get(), nact, mask, g->fwv_perm.get(),
+        LDS_LAUNCH(perm_from_keys_kernel, grid_for(nact, blk), blk, 0, s, rk.get(), nact, mask, perm.get(),
                    g->fwv_pos.get());
     }
+    g->fwv_perm = std::move(perm);
+}
+
+void ensure_fw_view(lds_graph* g) {
+    if (g->fwv_built) return;
+    ensure_fw_ranks(g);
+    cudaStream_t s = g->stream;
+    const int32_t nact = g->nact;
+    const int64_t m = g->m;
+    const int blk = 256;
     g->fwv_col.alloc(std::max<int64_t>(m, 1), s);
     g->fwv_chunk_nz0.alloc(std::max<int64_t>((m + 31) / 32, 1), s);
     g->fwv_edge.alloc(std::max<int64_t>(m, 1), s);
@@ -723,10 +643,8 @@ bool run_edge_fw_oriented(lds_graph* g, int N, lds_precision p, bool want_w, boo
     // 32-bit words: every scaled load below 2^32 and per-block hot counts below 2^16
     extern int g_fw_variant;
     // variant 3 keeps the row endpoints' counts inside the pass; variant 4 counts them
-    // in the vertex update but launches pass and update once per iteration; the
-    // default runs many iterations per cooperative launch
+    // in the vertex update
     const bool rows = g_fw_variant != 3;
-    const bool coop = g_fw_variant == 0 || g_fw_variant == 5 || g_fw_variant == 6;
     bool use32 = g_fw_variant != 2 && maxdeg < 65536 && (p == LDS_FP32 || (unsigned __int128)maxdeg * (unsigned __int128)Dn < ((unsigned __int128)1 << 32));
     if (!use32) {
         if (p == LDS_EXACT) {
@@ -759,10 +677,6 @@ bool run_edge_fw_oriented(lds_graph* g, int N, lds_precision p, bool want_w, boo
         if (nact)
             LDS_LAUNCH(oword_init_kernel, grid_for(nact, blk), blk, 0, s, g->rowptr.get(), g->fwv_perm.get(), nact, fp32,
                        w32.get(), r32.get());
-        LDS_CUDA(cudaFuncSetAttribute(fw_coop32_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)OP32_SMEM));
-        LDS_CUDA(cudaFuncSetAttribute(fw_coop32_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)OP32_SMEM));
         LDS_CUDA(cudaFuncSetAttribute(fw_opass32_kernel<OP_UNROLL, float, true>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OP32_SMEM));
         LDS_CUDA(cudaFuncSetAttribute(fw_opass32_kernel<OP_UNROLL, uint32_t, true>,
@@ -784,60 +698,7 @@ bool run_edge_fw_oriented(lds_graph* g, int N, lds_precision p, bool want_w, boo
     int stored = 0;
     int64_t first_i = 1;
     int64_t last_plane = 0;
-    if (use32 && coop && nchunks) {
-        int per_sm = 0;
-        if (fp32) LDS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fw_coop32_kernel<float>, OP_THREADS,
-                                                                         OP32_SMEM));
-        else LDS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fw_coop32_kernel<uint32_t>, OP_THREADS,
-                                                                    OP32_SMEM));
-        LDS_REQUIRE(per_sm >= 1, LDS_ECUDA, "fw: the cooperative pass cannot be resident");
-        g->pass_kernel = "fw_coop32_kernel";
-        const unsigned cgrid =
-            kCoopChunksPerBlock > 0
-                ? (unsigned)std::max<int64_t>(
-                      1, std::min<int64_t>(grid, (nchunks + kCoopChunksPerBlock - 1) / kCoopChunksPerBlock))
-                : grid;
-        DevBuf<uint32_t> hglob(((nhot + 1) >> 1) + 1, s);
-        LDS_CUDA(cudaMemsetAsync(hglob.get(), 0, (((nhot + 1) >> 1) + 1) * sizeof(uint32_t), s));
-        int i = 1;
-        while (i <= N) {
-            int32_t kk = std::min(K - stored, N - i + 1);
-            uint32_t* pl = planes.get() + (int64_t)stored * nchunks;
-            const int32_t* pcol = g->fwv_col.get();
-            const int32_t* pz = g->fwv_chunk_nz0.get();
-            const int32_t* pnz = g->fwv_nzrow.get();
-            const int32_t* pperm = g->fwv_perm.get();
-            const int32_t* prow = g->fwv_rowptr.get();
-            int32_t* pcnt = cnt.get();
-            int64_t nsl = m, nch = nchunks;
-            int32_t nh = nhot, na = nact, i0 = i;
-            void* wp = fp32 ? (void*)r32.get() : (void*)w32.get();
-            uint32_t* hg = hglob.get();
-            void* args[] = {(void*)&pcol, (void*)&pz, (void*)&pnz, (void*)&nsl, (void*)&nch, (void*)&wp, (void*)&pperm,
-                            (void*)&nh, (void*)&pcnt, (void*)&prow, (void*)&pl, (void*)&na, (void*)&i0, (void*)&kk,
-                            (void*)&hg};
-            timer.start(s);
-            if (fp32)
-                LDS_CUDA(cudaLaunchCooperativeKernel((void*)fw_coop32_kernel<float>, dim3(cgrid), dim3(OP_THREADS),
-                                                     args, OP32_SMEM, s));
-            else
-                LDS_CUDA(cudaLaunchCooperativeKernel((void*)fw_coop32_kernel<uint32_t>, dim3(cgrid), dim3(OP_THREADS),
-                                                     args, OP32_SMEM, s));
-            g_launches.fetch_add(1, std::memory_order_relaxed);
-            timer.stop(s, kk);
-            stored += kk;
-            i += kk;
-            if (stored == K || i > N) {
-                fold_planes(planes.get(), stored, nchunks, m, first_i, 2, W.get(), s);
-                last_plane = stored - 1;
-                if (i <= N) {
-                    stored = 0;
-                    first_i = i;
-                }
-            }
-        }
-    }
-    for (int i = (use32 && coop && nchunks) ? N + 1 : 1; i <= N; ++i) {
+    for (int i = 1; i <= N; ++i) {
         uint32_t* plane = planes.get() + (int64_t)stored * nchunks;
         if (nchunks) {
             const float gam = 2.0f / (float)(i + 2);

@@ -14,7 +14,7 @@
 // larger id; exact R <- R + 2(i+1) c, or binary32 r <- (1 - gamma) r + gamma c with
 // gamma = 2 / (i + 2) and each operation rounded on its own.
 //
-// An iteration here is latency: the grid-wide pass (fw_coop32_kernel) pays two grid
+// An iteration here is latency: the grid-wide pass (fw_quad_kernel and before it one slot a lane) pays two grid
 // barriers, a flush of shared counts and gathers from L2 whatever the size, and its
 // working set would fit the chip's registers many times over.  What is left is the
 // barrier, the copy of the load words (4 B per vertex and CTA, from L2) and about 25

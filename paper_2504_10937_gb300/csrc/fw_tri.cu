@@ -2,25 +2,30 @@
 //
 // Layout (the "triangle view", built once per graph).  Vertices are relabelled by
 // triangle count, descending.  T is sorted by (a, b, c), so the triangles of one pair
-// (a, b) are consecutive: a group.  Only c is stored per triangle, four to a quad,
-// every group padded to whole quads; bit 31 of a quad's first c marks the first quad
-// of a group, and tv_grp holds the group's (a, b).  tv_chunk_g0 is the group of the
-// first quad of each 32-quad chunk.
+// (a, b) are consecutive: a group.  Only c is stored per triangle, four to a quad;
+// bit 31 of a quad's first c marks the first quad of a group, and a list holds the
+// groups' (a, b).  Triangles whose three vertices are all among the hot ones (those
+// whose loads and counters fit shared memory) come first, the others after them, each
+// part with its own groups, padded to whole quads: the hot part, most of a skewed
+// graph's triangles, then needs no test of where a vertex lives.
 //
-// Pass.  A warp takes a chunk, a lane a quad.  The group's candidate among a and b
+// Pass.  A warp takes 32 quads, a lane one.  The group's candidate among a and b
 // (the smaller load, ties to b) is decided once for the quad; a triangle goes to c
 // when its load is not larger, else to that candidate: the lowest-load member, ties
-// to the larger id.  The loads of the highest-count vertices are staged in shared
-// memory with counters beside them; the receipts of a and b are added once per group
-// segment (bit-sliced popcounts over the segment's lanes), those of c one by one.
-// Two choice bits per triangle are four ballot words each per chunk: plane 0, b took
-// it; plane 1, c took it.  Many iterations (pass, grid barrier, vertex update, grid
-// barrier) run in one cooperative launch.  The update also keeps the exact loads
-// R = D r of the weights that the choices make: R += 6(i+1) receipts, whatever the
-// arithmetic of r.
+// to the larger id.  The receipts of a and b are added once per group segment (its
+// places that c did not win), those of c one by one.  Two choice bits per triangle
+// are four ballot words each per chunk: plane 0, b took it; plane 1, c took it.  Many
+// iterations (pass, grid barrier, vertex update, grid barrier) run in one cooperative
+// launch.  The update also keeps the exact loads R = D r of the weights that the
+// choices make: R += 6(i+1) receipts, whatever the arithmetic of r.
 //
-// What bounds it: 4 B of c per triangle from HBM when they exceed L2, about 80 warp
-// instructions per 128 triangles, and the shared atomics of the c receipts.
+// What bounds it: 4 B of c per triangle from HBM when they exceed L2, the warp
+// instructions of a chunk, and the shared-memory gathers and atomics of c.  Per
+// iteration on R-MAT scale 18 (84.6M triangles, binary32, GB300): 0.38 ms with one
+// thread per triangle and global atomics, 0.20 ms with quads whose every access
+// chose between shared and global memory (210 instructions a chunk), 0.17 ms with the
+// two parts (a chunk then waited 2,000 cycles for its groups' (a, b)), 0.134 ms with
+// the fetches a chunk and two ahead.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -38,8 +43,8 @@ namespace cg = cooperative_groups;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int TQ_THREADS = 1024;
 constexpr int TQ_CHUNK = 32;                     // quads of a warp step
-constexpr int32_t TQ_NONE = 0x7fffffff;          // padding (no vertex has this id)
 constexpr size_t TQ_SMEM = 224 * 1024;
+constexpr int32_t TQ_HOT = (int32_t)(TQ_SMEM / 8) - 8;     // hot ids with 4-byte loads: 4 B and a 4 B counter
 
 __device__ __forceinline__ unsigned lanes_le(int lane) { return lane == 31 ? FULL : (2u << lane) - 1u; }
 
@@ -74,63 +79,97 @@ __global__ void tv_rank_kernel(const uint64_t* key, int32_t nact, int32_t* perm,
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nact; p += stride) {
         const int32_t x = (int32_t)(key[p] & 0xffffffffu);
         perm[p] = x;
-        rank[x] = (int32_t)p;
+        rank[x] = (int32_t)p + 1;                // id 0 is padding
         count[p] = 0xffffffffu - (uint32_t)(key[p] >> 32);
     }
 }
 
-// bit t of start: triangle t begins a group
-__global__ void tv_start_kernel(const int32_t* ta, const int32_t* tb, int64_t nt, uint32_t* start, int32_t* cnt) {
+// bit t of start: triangle t begins a group; of hot: its vertices all have ids below nhot
+__global__ void tv_start_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt, const int32_t* rank,
+                                int32_t nhot, uint32_t* start, uint32_t* hot, int32_t* scnt, int32_t* hcnt) {
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5, nw = (nt + 31) >> 5;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw; w += nwarps) {
         const int64_t t = (w << 5) + lane;
-        const bool st = t < nt && (t == 0 || ta[t] != ta[t - 1] || tb[t] != tb[t - 1]);
-        const unsigned b = __ballot_sync(FULL, st);
+        bool st = false, h = false;
+        if (t < nt) {
+            const int32_t a = ta[t], b = tb[t];
+            st = t == 0 || a != ta[t - 1] || b != tb[t - 1];
+            h = rank[a] < nhot && rank[b] < nhot && rank[tc[t]] < nhot;
+        }
+        const unsigned sb = __ballot_sync(FULL, st), hb = __ballot_sync(FULL, h);
         if (lane == 0) {
-            start[w] = b;
-            cnt[w] = __popc(b);
+            start[w] = sb;
+            hot[w] = hb;
+            scnt[w] = __popc(sb);
+            hcnt[w] = __popc(hb);
         }
     }
 }
 
-__global__ void tv_group_kernel(const int32_t* ta, const int32_t* tb, int64_t nt, const uint32_t* start,
-                                const int64_t* base, const int32_t* rank, int64_t* gstart, int2* grp, int64_t ng) {
+__global__ void tv_group_kernel(int64_t nt, const uint32_t* start, const int64_t* sbase, int64_t* gstart, int64_t ng) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride) {
         const uint32_t b = start[t >> 5];
         if (!((b >> (t & 31)) & 1u)) continue;
-        const int64_t g = base[t >> 5] + __popc(b & ((1u << (t & 31)) - 1u));
+        const int64_t g = sbase[t >> 5] + __popc(b & ((1u << (t & 31)) - 1u));
         gstart[g] = t;
-        grp[g] = make_int2(rank[ta[t]], rank[tb[t]]);
         if (g == 0) gstart[ng] = nt;
     }
 }
 
-__global__ void tv_quads_kernel(const int64_t* gstart, int64_t ng, int32_t* nq) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g <= ng; g += stride)
-        nq[g] = g < ng ? (int32_t)((gstart[g + 1] - gstart[g] + 3) >> 2) : 0;
+// hot triangles before t
+__device__ __forceinline__ int64_t hot_before(int64_t t, int64_t nt, const uint32_t* hot, const int64_t* hbase) {
+    if (t >= nt) t = nt;
+    const int64_t w = t >> 5;
+    return (t & 31) ? hbase[w] + __popc(hot[w] & ((1u << (t & 31)) - 1u)) : hbase[w];
 }
 
-__global__ void tv_fill_none_kernel(int32_t* c, int64_t k) {
+// quads of each group in the hot part and in the other, and whether it has any
+__global__ void tv_quads_kernel(const int64_t* gstart, int64_t ng, int64_t nt, const uint32_t* hot, const int64_t* hbase,
+                                int32_t* qh, int32_t* qx, int32_t* anyh, int32_t* anyx) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += stride) c[i] = TQ_NONE;
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g <= ng; g += stride) {
+        int64_t h = 0, x = 0;
+        if (g < ng) {
+            h = hot_before(gstart[g + 1], nt, hot, hbase) - hot_before(gstart[g], nt, hot, hbase);
+            x = gstart[g + 1] - gstart[g] - h;
+        }
+        qh[g] = (int32_t)((h + 3) >> 2);
+        qx[g] = (int32_t)((x + 3) >> 2);
+        anyh[g] = h > 0;
+        anyx[g] = x > 0;
+    }
 }
 
-__global__ void tv_fill_kernel(const int32_t* tc, int64_t nt, const uint32_t* start, const int64_t* base,
-                               const int64_t* gstart, const int64_t* qstart, const int32_t* rank, int32_t* c,
-                               uint32_t* qt, int32_t* chunk_g0) {
+struct TvFill {
+    const uint32_t *start, *hot;
+    const int64_t *sbase, *hbase, *gstart;
+    const int64_t *qh, *qx, *gh, *gx;     // per group: first quad and index among the part's groups
+    int64_t xquad, xgrp;                  // first quad and group of the second part
+    const int32_t* rank;
+    int32_t* c;
+    uint32_t* it;
+    int32_t* chunk_g0;
+    int2* grp;
+};
+
+__global__ void tv_fill_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt, TvFill F) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride) {
-        const uint32_t b = start[t >> 5];
-        const int64_t g = base[t >> 5] + __popc(b & lanes_le((int)(t & 31))) - 1;
-        const int64_t off = t - gstart[g], q = qstart[g] + (off >> 2);
-        c[4 * q + (off & 3)] = rank[tc[t]] | (off == 0 ? (int32_t)0x80000000 : 0);
-        if ((off & 3) == 0) {
-            qt[q] = (uint32_t)t;
-            if ((q & (TQ_CHUNK - 1)) == 0) chunk_g0[q / TQ_CHUNK] = (int32_t)g;
-        }
+        const int64_t w = t >> 5;
+        const int l = (int)(t & 31);
+        const int64_t g = F.sbase[w] + __popc(F.start[w] & lanes_le(l)) - 1;
+        const int64_t gs = F.gstart[g];
+        const int64_t hb = hot_before(t, nt, F.hot, F.hbase) - hot_before(gs, nt, F.hot, F.hbase);
+        const bool h = (F.hot[w] >> l) & 1u;
+        const int64_t off = h ? hb : (t - gs) - hb;
+        const int64_t q = (h ? F.qh[g] : F.xquad + F.qx[g]) + (off >> 2);
+        const int64_t gi = h ? F.gh[g] : F.xgrp + F.gx[g];
+        F.c[4 * q + (off & 3)] = F.rank[tc[t]] | (off == 0 ? (int32_t)0x80000000 : 0);
+        F.it[4 * q + (off & 3)] = (uint32_t)t;
+        if (off == 0) F.grp[gi] = make_int2(F.rank[ta[t]], F.rank[tb[t]]);
+        if ((off & 3) == 0 && (q & (TQ_CHUNK - 1)) == 0) F.chunk_g0[q / TQ_CHUNK] = (int32_t)gi;
     }
 }
 
@@ -140,104 +179,106 @@ struct TqArgs {
     const int4* c;               // [nq padded to whole chunks]
     const int32_t* chunk_g0;
     const int2* grp;
-    int64_t nchunks;
-    int32_t nact, nhot;
-    void* load;                  // [nact] loads by rank: float, or R as int64 (exact)
-    int64_t* R;                  // [nact] exact loads of the weights (binary32 only; exact has them in load)
-    uint32_t* cnt;               // [nact] receipts, zero between iterations
+    int64_t nchunks, hchunks;    // chunks in all; of the hot part (its ids all below nhot), which comes first
+    int32_t nact, nhot;          // vertices 1 .. nact by rank; the first nhot ids are staged
+    void* load;                  // [nact + 1] loads by rank: float, or R as int64 (exact)
+    int64_t* R;                  // [nact + 1] exact loads of the weights (binary32 only; exact has them in load)
+    uint32_t* cnt;               // [nact + 1] receipts, zero between iterations
     uint4* planes;               // per iteration: [nchunks] words of plane 0, then of plane 1
     int32_t i_first, K;
 };
 
+// Id 0 is the padding of a quad: its load -1 lies below every load, so it always
+// "wins" its place, receives nothing, and needs no test of its own.
 template <class L>
 __global__ void __launch_bounds__(TQ_THREADS, 1) fw_tri_quad_kernel(const TqArgs A) {
     cg::grid_group grid = cg::this_grid();
     extern __shared__ __align__(16) unsigned char smem[];
-    L* hl = reinterpret_cast<L*>(smem);
-    uint32_t* hc = reinterpret_cast<uint32_t*>(smem + (((size_t)A.nhot * sizeof(L) + 15) & ~(size_t)15));
+    L* const hl = reinterpret_cast<L*>(smem);
+    uint32_t* const hc = reinterpret_cast<uint32_t*>(smem + (((size_t)A.nhot * sizeof(L) + 15) & ~(size_t)15));
     L* const load = reinterpret_cast<L*>(A.load);
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + tid, nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int64_t warp = gtid >> 5, nwarps = nthreads >> 5;
-    const int32_t nhot = A.nhot, nact = A.nact;
+    const uint32_t warp = (uint32_t)(gtid >> 5), nwarps = (uint32_t)(nthreads >> 5), nch = (uint32_t)A.nchunks;
+    const uint32_t nhot = (uint32_t)A.nhot, hch = (uint32_t)A.hchunks;
     const unsigned le = lanes_le(lane);
     for (int32_t it = 0; it < A.K; ++it) {
         const int32_t i = A.i_first + it;
-        for (int32_t j = tid; j < nhot; j += TQ_THREADS) {
+        for (uint32_t j = tid; j < nhot; j += TQ_THREADS) {
             hl[j] = __ldcg(load + j);
             hc[j] = 0;
         }
         __syncthreads();
-        uint4* p0 = A.planes + 2 * (int64_t)it * A.nchunks;
-        uint4* p1 = p0 + A.nchunks;
-        int4 cn = make_int4(TQ_NONE, TQ_NONE, TQ_NONE, TQ_NONE);
-        int32_t gn = 0;
-        if (warp < A.nchunks) {
-            cn = __ldg(A.c + warp * TQ_CHUNK + lane);
-            gn = __ldg(A.chunk_g0 + warp);
-        }
-        for (int64_t ch = warp; ch < A.nchunks; ch += nwarps) {
-            const int4 c4 = cn;
-            const int32_t g0 = gn;
-            if (ch + nwarps < A.nchunks) {
-                cn = __ldg(A.c + (ch + nwarps) * TQ_CHUNK + lane);
-                gn = __ldg(A.chunk_g0 + ch + nwarps);
-            }
+        uint4* const p0 = A.planes + 2 * (int64_t)it * A.nchunks;
+        uint4* const p1 = p0 + A.nchunks;
+        // three chunks in flight: the groups' (a, b) of this one have arrived, the next one's
+        // are fetched (its c have arrived), the c of the one after are fetched
+        auto fetch_c = [&](uint32_t ch) { return ch < nch ? __ldg(A.c + (int64_t)ch * TQ_CHUNK + lane) : make_int4(0, 0, 0, 0); };
+        auto fetch_g = [&](uint32_t ch) { return ch < nch ? __ldg(A.chunk_g0 + ch) : 0; };
+        auto fetch_ab = [&](const int4& c, int32_t g0) {
+            const unsigned f = __ballot_sync(FULL, c.x < 0);
+            return __ldg(A.grp + (g0 + __popc(f & le) - (int)(f & 1u)));
+        };
+        int4 ca = fetch_c(warp), cb = fetch_c(warp + nwarps);
+        int32_t gb = fetch_g(warp + nwarps);
+        int2 aba = fetch_ab(ca, fetch_g(warp));
+        // one chunk; ld and add reach a vertex's load and counter
+        auto chunk = [&](uint32_t ch, auto&& ld, auto&& add) {
+            const int4 c4 = ca, cc = fetch_c(ch + 2 * nwarps);
+            const int32_t gc = fetch_g(ch + 2 * nwarps);
+            const int2 ab = aba, abb = fetch_ab(cb, gb);
             const unsigned f = __ballot_sync(FULL, c4.x < 0);
-            const int2 ab = __ldg(A.grp + (g0 + __popc(f & le) - (int)(f & 1u)));
-            const int32_t c[4] = {c4.x & 0x7fffffff, c4.y, c4.z, c4.w};
+            const uint32_t c[4] = {(uint32_t)c4.x & 0x7fffffffu, (uint32_t)c4.y, (uint32_t)c4.z, (uint32_t)c4.w};
             L rc[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int32_t cj = c[j] < nact ? c[j] : 0;
-                rc[j] = cj < nhot ? hl[cj] : __ldcg(load + cj);
-            }
-            const L ra = ab.x < nhot ? hl[ab.x] : __ldcg(load + ab.x);
-            const L rb = ab.y < nhot ? hl[ab.y] : __ldcg(load + ab.y);
+            for (int j = 0; j < 4; ++j) rc[j] = ld(c[j]);
+            const L ra = ld((uint32_t)ab.x), rb = ld((uint32_t)ab.y);
             const bool to_a = ra < rb;
             const L val = to_a ? ra : rb;
-            const int32_t win = to_a ? ab.x : ab.y;
             const unsigned bb = __ballot_sync(FULL, !to_a);
-            unsigned w0[4], w1[4];
-            int k = 0;                           // triangles of the quad that a or b takes
+            unsigned w1[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const bool ok = c[j] < nact;
-                const bool cw = ok && !(val < rc[j]);
-                const unsigned okm = __ballot_sync(FULL, ok);
+                const bool cw = !(val < rc[j]);
                 w1[j] = __ballot_sync(FULL, cw);
-                w0[j] = okm & bb & ~w1[j];
-                k += ok && !cw;
-                if (cw) {
-                    if (c[j] < nhot) atomicAdd(hc + c[j], 1u);
-                    else atomicAdd(A.cnt + c[j], 1u);
-                }
+                if (cw && c[j] != 0) add(c[j], 1u);
             }
             if (lane == 0) {
-                __stcs(p0 + ch, make_uint4(w0[0], w0[1], w0[2], w0[3]));
+                __stcs(p0 + ch, make_uint4(bb & ~w1[0], bb & ~w1[1], bb & ~w1[2], bb & ~w1[3]));
                 __stcs(p1 + ch, make_uint4(w1[0], w1[1], w1[2], w1[3]));
             }
-            // receipts of the group segment: k summed over its lanes by bits
-            const unsigned k0 = __ballot_sync(FULL, k & 1), k1 = __ballot_sync(FULL, k & 2), k2 = __ballot_sync(FULL, k & 4);
-            if (lane == 0 || ((f >> lane) & 1u)) {
+            // receipts of a or b in the group segment: its places that c did not win
+            if (lane == 0 || c4.x < 0) {
                 const unsigned above = f & ~le;
                 const unsigned seg = (FULL << lane) & (above ? (above & (0u - above)) - 1u : FULL);
-                const unsigned n = __popc(k0 & seg) + 2 * __popc(k1 & seg) + 4 * __popc(k2 & seg);
-                if (n) {
-                    if (win < nhot) atomicAdd(hc + win, n);
-                    else atomicAdd(A.cnt + win, n);
-                }
+                const unsigned n = 4 * __popc(seg) - (__popc(w1[0] & seg) + __popc(w1[1] & seg) + __popc(w1[2] & seg) +
+                                                      __popc(w1[3] & seg));
+                if (n) add((uint32_t)(to_a ? ab.x : ab.y), n);
             }
-        }
+            ca = cb;
+            cb = cc;
+            gb = gc;
+            aba = abb;
+        };
+        uint32_t ch = warp;
+        for (; ch < hch; ch += nwarps)
+            chunk(ch, [&](uint32_t x) { return hl[x]; }, [&](uint32_t x, uint32_t v) { atomicAdd(hc + x, v); });
+        for (; ch < nch; ch += nwarps)
+            chunk(
+                ch, [&](uint32_t x) { return *((x < nhot ? hl : load) + x); },
+                [&](uint32_t x, uint32_t v) {
+                    if (x < nhot) atomicAdd(hc + x, v);
+                    else atomicAdd(A.cnt + x, v);
+                });
         __syncthreads();
-        for (int32_t j = tid; j < nhot; j += TQ_THREADS) {
+        for (uint32_t j = tid; j < nhot; j += TQ_THREADS) {
             const uint32_t v = hc[j];
             if (v) atomicAdd(A.cnt + j, v);
         }
         grid.sync();
         const float gam = __fdiv_rn(2.0f, (float)(i + 2));
         const float om = __fsub_rn(1.0f, gam);
-        for (int64_t p = gtid; p < nact; p += nthreads) {
+        for (int64_t p = 1 + gtid; p <= A.nact; p += nthreads) {
             const uint32_t n = __ldcg(A.cnt + p);
             if (n) A.cnt[p] = 0;
             const int64_t grow = 6 * (int64_t)(i + 1) * (int64_t)n;
@@ -254,91 +295,33 @@ __global__ void __launch_bounds__(TQ_THREADS, 1) fw_tri_quad_kernel(const TqArgs
 
 __global__ void tq_init_kernel(const uint32_t* count, int32_t nact, float* r32, int64_t* R) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nact; p += stride) {
-        R[p] = 2 * (int64_t)count[p];            // R0 = D_0 t / 3, D_0 = 6
-        if (r32) r32[p] = __fdiv_rn((float)count[p], 3.0f);
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= nact; p += stride) {
+        R[p] = p ? 2 * (int64_t)count[p - 1] : -1;           // R0 = D_0 t / 3, D_0 = 6
+        if (r32) r32[p] = p ? __fdiv_rn((float)count[p - 1], 3.0f) : -1.0f;
     }
 }
 
-// ---------------------------------------------------------------- fold
-
-// 32 x 32 bit transpose over a warp: lane l gives row l and receives column l
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-    uint32_t m = 0x0000ffffu;
-#pragma unroll
-    for (int s = 16; s; s >>= 1) {
-        const uint32_t y = __shfl_xor_sync(FULL, x, s);
-        x = (lane & s) ? ((x & ~m) | ((y >> s) & m)) : ((x & m) | ((y << s) & ~m));
-        m ^= m << (s >> 1);
-    }
-    return x;
-}
-
-// sum over set bits j of (first + j), by bits of j
-__device__ __forceinline__ uint32_t weighted(uint32_t w, uint32_t first) {
-    return first * __popc(w) + __popc(w & 0xaaaaaaaau) + 2 * __popc(w & 0xccccccccu) + 4 * __popc(w & 0xf0f0f0f0u) +
-           8 * __popc(w & 0xff00ff00u) + 16 * __popc(w & 0xffff0000u);
-}
-
-// W of b and of c grow by 6(i+1) per set bit of their plane.  A block takes 8 chunks
-// (32 words of each plane), 32 iterations at a time: the words of 32 iterations are
-// transposed in the warp, so a lane holds one triangle's 32 choices and adds their
-// weights by popcounts.  Word j, bit l of a chunk is item 4 l + j.
-constexpr int TF_CHUNKS = 8;
-__global__ void __launch_bounds__(1024) fw_tri_fold_kernel(const uint32_t* __restrict__ planes, int nplanes,
-                                                           int64_t nchunks, int64_t i_first, uint32_t* Wb, uint32_t* Wc) {
-    __shared__ uint32_t tile[2][32][33];
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const int64_t words = 4 * nchunks;
-    for (int64_t c0 = (int64_t)blockIdx.x * TF_CHUNKS; c0 < nchunks; c0 += (int64_t)gridDim.x * TF_CHUNKS) {
-        uint32_t ab = 0, ac = 0;
-        for (int k0 = 0; k0 < nplanes; k0 += 32) {
-            const int k = k0 + w;
-            const int64_t at = 4 * c0 + lane;
-            const bool in = k < nplanes && at < words;
-            tile[0][w][lane] = in ? __ldcs(planes + 2 * (int64_t)k * words + at) : 0u;
-            tile[1][w][lane] = in ? __ldcs(planes + (2 * (int64_t)k + 1) * words + at) : 0u;
-            __syncthreads();
-            // warp w takes word w: row l of the matrix is iteration l
-            const uint32_t hb = transpose32(tile[0][lane][w], lane), hcc = transpose32(tile[1][lane][w], lane);
-            const uint32_t first = (uint32_t)(i_first + k0 + 1);
-            ab += 6u * weighted(hb, first);
-            ac += 6u * weighted(hcc, first);
-            __syncthreads();
-        }
-        // word w is word (w & 3) of chunk c0 + (w >> 2)
-        const int64_t ch = c0 + (w >> 2);
-        if (ch < nchunks) {
-            const int64_t item = ch * 128 + 4 * lane + (w & 3);
-            Wb[item] += ab;
-            Wc[item] += ac;
-        }
-    }
-}
+// ---------------------------------------------------------------- outputs
 
 // weights and last choices in triangle order
-__global__ void tq_output_kernel(const int32_t* c, const uint32_t* qt, int64_t nq, int32_t nact, const uint32_t* Wb,
+__global__ void tq_output_kernel(const int32_t* c, const uint32_t* it, int64_t items, const uint32_t* Wb,
                                  const uint32_t* Wc, uint32_t D3, int64_t* W, const uint32_t* plane0,
                                  const uint32_t* plane1, uint8_t* last) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += stride) {
-        const int64_t t0 = qt[q];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t item = 4 * q + j;
-            if ((c[item] & 0x7fffffff) >= nact) break;
-            const uint32_t b = Wb[item] + 2u, cc = Wc[item] + 2u;      // W0 = D_0 / 3
-            W[3 * (t0 + j)] = (int64_t)(D3 - b - cc);
-            W[3 * (t0 + j) + 1] = (int64_t)b;
-            W[3 * (t0 + j) + 2] = (int64_t)cc;
-            if (last) {
-                uint32_t col = 2;
-                if (plane0) {
-                    const int64_t word = 4 * (q >> 5) + j;
-                    col = ((plane0[word] >> (q & 31)) & 1u) | (((plane1[word] >> (q & 31)) & 1u) << 1);
-                }
-                last[t0 + j] = (uint8_t)col;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += stride) {
+        if ((c[i] & 0x7fffffff) == 0) continue;
+        const int64_t t = it[i];
+        const uint32_t b = Wb[i] + 2u, cc = Wc[i] + 2u;      // W0 = D_0 / 3
+        W[3 * t] = (int64_t)(D3 - b - cc);
+        W[3 * t + 1] = (int64_t)b;
+        W[3 * t + 2] = (int64_t)cc;
+        if (last) {
+            uint32_t col = 2;
+            if (plane0) {
+                const int64_t q = i >> 2, word = 4 * (q >> 5) + (i & 3);
+                col = ((plane0[word] >> (q & 31)) & 1u) | (((plane1[word] >> (q & 31)) & 1u) << 1);
             }
+            last[t] = (uint8_t)col;
         }
     }
 }
@@ -348,8 +331,8 @@ __global__ void tq_loads_out_kernel(const int32_t* perm, int32_t nact, const int
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nact; p += stride) {
         const int32_t x = perm[p];
-        R_int[x] = R[p];
-        r_int[x] = r32 ? (double)r32[p] : (double)R[p] / D3;
+        R_int[x] = R[p + 1];
+        r_int[x] = r32 ? (double)r32[p + 1] : (double)R[p + 1] / D3;
     }
 }
 
@@ -375,25 +358,38 @@ static void ensure_tri_view(lds_graph* g) {
     LDS_LAUNCH(tv_rank_kernel, grid_for(nact, blk), blk, 0, s, key.get(), nact, g->tv_perm.get(), rank.get(),
                g->tv_count.get());
     const int64_t nw = (nt + 31) / 32;
-    DevBuf<uint32_t> start(nw, s);
-    DevBuf<int32_t> wc(nw, s);
-    DevBuf<int64_t> base(nw, s);
-    LDS_LAUNCH(tv_start_kernel, grid_for(nt, blk), blk, 0, s, g->ta.get(), g->tb.get(), nt, start.get(), wc.get());
-    const int64_t ng = exclusive_scan_i32_to_i64(wc.get(), base.get(), nw, s);
-    DevBuf<int64_t> gstart(ng + 1, s), qstart(ng + 1, s);
-    DevBuf<int32_t> nqs(ng + 1, s);
-    g->tv_grp.alloc(ng, s);
-    LDS_LAUNCH(tv_group_kernel, grid_for(nt, blk), blk, 0, s, g->ta.get(), g->tb.get(), nt, start.get(), base.get(),
-               rank.get(), gstart.get(), g->tv_grp.get(), ng);
-    LDS_LAUNCH(tv_quads_kernel, grid_for(ng + 1, blk), blk, 0, s, gstart.get(), ng, nqs.get());
-    g->tv_nq = exclusive_scan_i32_to_i64(nqs.get(), qstart.get(), ng + 1, s);
-    const int64_t chunks = (g->tv_nq + TQ_CHUNK - 1) / TQ_CHUNK;
-    DevBuf<int32_t> c(4 * TQ_CHUNK * chunks, s);
-    g->tv_qt.alloc(g->tv_nq, s);
-    g->tv_chunk_g0.alloc(chunks, s);
-    LDS_LAUNCH(tv_fill_none_kernel, grid_for(4 * TQ_CHUNK * chunks, blk), blk, 0, s, c.get(), 4 * TQ_CHUNK * chunks);
-    LDS_LAUNCH(tv_fill_kernel, grid_for(nt, blk), blk, 0, s, g->tc.get(), nt, start.get(), base.get(), gstart.get(),
-               qstart.get(), rank.get(), c.get(), g->tv_qt.get(), g->tv_chunk_g0.get());
+    DevBuf<uint32_t> start(nw, s), hot(nw, s);
+    DevBuf<int32_t> sc(nw, s), hc(nw + 1, s);
+    DevBuf<int64_t> sbase(nw, s), hbase(nw + 1, s);
+    LDS_CUDA(cudaMemsetAsync(hc.get() + nw, 0, sizeof(int32_t), s));
+    LDS_LAUNCH(tv_start_kernel, grid_for(nt, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), nt, rank.get(),
+               TQ_HOT, start.get(), hot.get(), sc.get(), hc.get());
+    exclusive_scan_i32_dev(hc.get(), hbase.get(), nw + 1, s);
+    const int64_t ng = exclusive_scan_i32_to_i64(sc.get(), sbase.get(), nw, s);
+    DevBuf<int64_t> gstart(ng + 1, s), qh(ng + 1, s), qx(ng + 1, s), gh(ng + 1, s), gx(ng + 1, s);
+    LDS_LAUNCH(tv_group_kernel, grid_for(nt, blk), blk, 0, s, nt, start.get(), sbase.get(), gstart.get(), ng);
+    int64_t nqh, nqx, ngh, ngx;
+    {
+        DevBuf<int32_t> a(ng + 1, s), b(ng + 1, s), c(ng + 1, s), d(ng + 1, s);
+        LDS_LAUNCH(tv_quads_kernel, grid_for(ng + 1, blk), blk, 0, s, gstart.get(), ng, nt, hot.get(), hbase.get(), a.get(),
+                   b.get(), c.get(), d.get());
+        nqh = exclusive_scan_i32_to_i64(a.get(), qh.get(), ng + 1, s);
+        nqx = exclusive_scan_i32_to_i64(b.get(), qx.get(), ng + 1, s);
+        ngh = exclusive_scan_i32_to_i64(c.get(), gh.get(), ng + 1, s);
+        ngx = exclusive_scan_i32_to_i64(d.get(), gx.get(), ng + 1, s);
+    }
+    g->tv_hchunks = (nqh + TQ_CHUNK - 1) / TQ_CHUNK;
+    g->tv_chunks = g->tv_hchunks + (nqx + TQ_CHUNK - 1) / TQ_CHUNK;
+    const int64_t items = 4 * TQ_CHUNK * g->tv_chunks;
+    DevBuf<int32_t> c(items, s);
+    g->tv_it.alloc(items, s);
+    g->tv_chunk_g0.alloc(g->tv_chunks, s);
+    g->tv_grp.alloc(ngh + ngx, s);
+    LDS_CUDA(cudaMemsetAsync(c.get(), 0, items * sizeof(int32_t), s));
+    TvFill F{start.get(),  hot.get(), sbase.get(), hbase.get(), gstart.get(), qh.get(), qx.get(),  gh.get(),
+             gx.get(),     g->tv_hchunks * TQ_CHUNK, ngh,       rank.get(),   c.get(),  g->tv_it.get(),
+             g->tv_chunk_g0.get(), g->tv_grp.get()};
+    LDS_LAUNCH(tv_fill_kernel, grid_for(nt, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), nt, F);
     g->tv_c = std::move(c);
 }
 
@@ -409,42 +405,43 @@ void run_tri_fw(lds_graph* g, int N, lds_precision p, bool want_last, PassTimer&
     if (want_last) g->fw_last.alloc(std::max<int64_t>(nt, 1), s);
     if (nt == 0) return;
     ensure_tri_view(g);
-    const int64_t nq = g->tv_nq, nchunks = (nq + TQ_CHUNK - 1) / TQ_CHUNK;
-    DevBuf<int64_t> R(nact, s);
-    DevBuf<float> r32(fp32 ? nact : 0, s);
-    DevBuf<uint32_t> cnt(nact, s);
-    LDS_CUDA(cudaMemsetAsync(cnt.get(), 0, nact * sizeof(uint32_t), s));
+    const int64_t nchunks = g->tv_chunks, items = 4 * TQ_CHUNK * nchunks;
+    DevBuf<int64_t> R((size_t)nact + 1, s);
+    DevBuf<float> r32(fp32 ? (size_t)nact + 1 : 0, s);
+    DevBuf<uint32_t> cnt((size_t)nact + 1, s);
+    LDS_CUDA(cudaMemsetAsync(cnt.get(), 0, ((size_t)nact + 1) * sizeof(uint32_t), s));
     LDS_LAUNCH(tq_init_kernel, grid_for(nact, blk), blk, 0, s, g->tv_count.get(), nact, r32.get(), R.get());
     const int K = planes_capacity(8 * nchunks, N);
     DevBuf<uint4> planes(std::max<int64_t>(1, 2 * (int64_t)K * nchunks), s);
-    DevBuf<uint32_t> Wb(128 * nchunks, s), Wc(128 * nchunks, s);
-    LDS_CUDA(cudaMemsetAsync(Wb.get(), 0, 128 * nchunks * sizeof(uint32_t), s));
-    LDS_CUDA(cudaMemsetAsync(Wc.get(), 0, 128 * nchunks * sizeof(uint32_t), s));
+    DevBuf<uint32_t> Wb(items, s), Wc(items, s);
+    LDS_CUDA(cudaMemsetAsync(Wb.get(), 0, items * sizeof(uint32_t), s));
+    LDS_CUDA(cudaMemsetAsync(Wc.get(), 0, items * sizeof(uint32_t), s));
     const void* fn = fp32 ? (const void*)fw_tri_quad_kernel<float> : (const void*)fw_tri_quad_kernel<int64_t>;
     LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TQ_SMEM));
     const size_t lsize = fp32 ? sizeof(float) : sizeof(int64_t);
-    const int32_t nhot = (int32_t)std::min<int64_t>(nact, (int64_t)((TQ_SMEM - 32) / (lsize + 4)));
+    const int32_t nhot =
+        (int32_t)std::min<int64_t>((int64_t)nact + 1, fp32 ? (int64_t)TQ_HOT : (int64_t)((TQ_SMEM - 32) / (lsize + 4)));
     const size_t smem = (((size_t)nhot * lsize + 15) & ~(size_t)15) + (size_t)nhot * 4;
+    // 64-bit loads stage fewer ids: unless that is all of them, every chunk takes the general form
+    const int64_t hchunks = fp32 || nhot == nact + 1 ? g->tv_hchunks : 0;
     // two chunks a warp at least: a block's staging and flush of the hot vertices is
     // shared by its passes over them
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms(), (nchunks + 63) / 64));
     int stored = 0;
     for (int i = 1; i <= N; i += stored) {
         stored = std::min(K, N - i + 1);
-        TqArgs A{reinterpret_cast<const int4*>(g->tv_c.get()), g->tv_chunk_g0.get(), g->tv_grp.get(), nchunks, nact, nhot,
+        TqArgs A{reinterpret_cast<const int4*>(g->tv_c.get()), g->tv_chunk_g0.get(), g->tv_grp.get(), nchunks, hchunks, nact, nhot,
                  fp32 ? (void*)r32.get() : (void*)R.get(), R.get(), cnt.get(), planes.get(), i, stored};
         void* args[] = {(void*)&A};
         timer.start(s);
         LDS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(TQ_THREADS), args, smem, s));
         g_launches.fetch_add(1, std::memory_order_relaxed);
         timer.stop(s, stored);
-        const int64_t fblocks = (nchunks + TF_CHUNKS - 1) / TF_CHUNKS;
-        LDS_LAUNCH(fw_tri_fold_kernel, (unsigned)std::min<int64_t>(fblocks, (int64_t)num_sms() * 16), 1024, 0, s,
-                   reinterpret_cast<const uint32_t*>(planes.get()), stored, nchunks, (int64_t)i, Wb.get(), Wc.get());
+        fold_quads(reinterpret_cast<const uint32_t*>(planes.get()), stored, nchunks, i, 6, Wb.get(), Wc.get(), s);
     }
     const int64_t D3 = 3 * (int64_t)(N + 1) * (N + 2);
     const uint32_t* last0 = N ? reinterpret_cast<const uint32_t*>(planes.get() + 2 * (int64_t)(stored - 1) * nchunks) : nullptr;
-    LDS_LAUNCH(tq_output_kernel, grid_for(nq, blk), blk, 0, s, g->tv_c.get(), g->tv_qt.get(), nq, nact, Wb.get(), Wc.get(),
+    LDS_LAUNCH(tq_output_kernel, grid_for(items, blk), blk, 0, s, g->tv_c.get(), g->tv_it.get(), items, Wb.get(), Wc.get(),
                (uint32_t)D3, g->fw_W.get(), last0, last0 ? last0 + 4 * nchunks : nullptr,
                want_last ? g->fw_last.get() : nullptr);
     LDS_LAUNCH(tq_loads_out_kernel, grid_for(nact, blk), blk, 0, s, g->tv_perm.get(), nact, R.get(), r32.get(), (double)D3,

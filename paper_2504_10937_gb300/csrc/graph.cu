@@ -349,9 +349,14 @@ void set_stream(lds_graph* g, cudaStream_t s) {
     g->tv_perm.s = s;
     g->tv_count.s = s;
     g->tv_c.s = s;
-    g->tv_qt.s = s;
+    g->tv_it.s = s;
     g->tv_chunk_g0.s = s;
     g->tv_grp.s = s;
+    g->fwq_c.s = s;
+    g->fwq_qs.s = s;
+    g->fwq_src.s = s;
+    g->fwq_qptr.s = s;
+    g->fwq_eid.s = s;
     g->fw_R.s = s;
     g->fw_r.s = s;
     g->fw_W.s = s;

@@ -52,13 +52,21 @@ struct lds_graph {
 
     // triangle FW view (lazy, fw_tri.cu): vertices ranked by (triangle count descending,
     // id ascending); the triangles of one (a, b) consecutive, c in quads
-    int64_t tv_nq = 0;
+    int64_t tv_chunks = 0, tv_hchunks = 0;     // 32-quad chunks in all, of the hot part
     lds::DevBuf<int32_t> tv_perm;      // [nact] rank -> internal id
     lds::DevBuf<uint32_t> tv_count;    // [nact] triangles of the vertex of each rank
-    lds::DevBuf<int32_t> tv_c;         // [4 tv_nq, padded to chunks] rank of c; bit 31: first quad of a group
-    lds::DevBuf<uint32_t> tv_qt;       // [tv_nq] triangle of each quad's first entry
-    lds::DevBuf<int32_t> tv_chunk_g0;  // group of the first quad of each 32-quad chunk
-    lds::DevBuf<int2> tv_grp;          // (a, b) of each group, as ranks
+    lds::DevBuf<int32_t> tv_c;         // [128 tv_chunks] 1 + rank of c, 0 padding; bit 31: first quad of a group
+    lds::DevBuf<uint32_t> tv_it;       // [128 tv_chunks] triangle of each entry
+    lds::DevBuf<int32_t> tv_chunk_g0;  // [tv_chunks] group of the first quad of each chunk
+    lds::DevBuf<int2> tv_grp;          // (a, b) of each group, as 1 + rank
+
+    // edge FW quad view (lazy, fw_quads.cu), in the ranks of fwv_perm
+    int64_t fwq_nq = 0;                // quads
+    lds::DevBuf<int32_t> fwq_c;        // [4 fwq_nq, padded to 32-quad chunks] 1 + rank of the target, 0 padding
+    lds::DevBuf<int32_t> fwq_src;      // [fwq_nq, padded] 1 + rank of each quad's row, 0 padding
+    lds::DevBuf<int32_t> fwq_qs;       // [fwq_nq] slot of each quad's first entry
+    lds::DevBuf<int32_t> fwq_qptr;     // [nact + 1] quads of the row of each rank
+    lds::DevBuf<uint32_t> fwq_eid;     // [m] 2 * canonical edge of a slot, + 1 when its lower endpoint is the row's
 
     // state of the most recent Frank-Wolfe run (internal ids), read by the later stages
     bool fw_valid = false;
@@ -95,8 +103,9 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
 // Copies r, R, W (and the last choices when asked) of the handle's state out.
 void copy_fw_state(lds_graph* g, lds_density d, lds_mem where, lds_fw_result* out);
 
-// Builds the FW view (see lds_graph) if not present.
+// Builds the FW view (see lds_graph) if not present; the ranks (fwv_perm, fwv_pos) alone.
 void ensure_fw_view(lds_graph* g);
+void ensure_fw_ranks(lds_graph* g);
 
 // Builds the vertex -> triangle incidence (ascending triangle order) if not present.
 void ensure_vertex_triangles(lds_graph* g);
