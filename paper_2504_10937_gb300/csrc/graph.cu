@@ -381,10 +381,12 @@ lds_status lds_create_graph(int32_t n, int64_t m, const int32_t* src, const int3
         LDS_REQUIRE(lds_device_count() > 0, LDS_ECUDA, "lds_create_graph: no CUDA device");
         lds_graph* g = new lds_graph();
         g->stream = (cudaStream_t)stream;
+        handle_created();
         try {
             build_graph(g, n, m, src, dst, where);
         } catch (...) {
             delete g;
+            handle_freed();
             throw;
         }
         *out = g;
@@ -396,6 +398,7 @@ void lds_free(lds_graph* g) {
     cudaStreamSynchronize(g->stream);
     delete g;
     cudaStreamSynchronize(nullptr);
+    handle_freed();
 }
 
 lds_status lds_graph_info(const lds_graph* g, lds_graph_info_t* info) {
