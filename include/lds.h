@@ -381,7 +381,9 @@ lds_status lds_batch_autotune(int32_t count, const lds_query* queries, int32_t* 
  * whether each one's graph is busy, and the free budget; -1 if none fits. */
 int32_t lds_debug_pick_next(int32_t nq, const int64_t* bytes, const uint8_t* graph_busy, int64_t free_bytes);
 
-/* Edge-density kernel choice for LDS_EXACT / LDS_FP32 (process-wide):
+/* Edge-density kernel choice (process-wide; LDS_FP64 has the resident form of 0
+ * for graphs that fit it, and one slot pass and one row-sum launch per iteration
+ * otherwise and under any other variant but 6):
  *   0  automatic: a graph of at most 65,536 active vertices whose symmetric
  *      CSR slots fit the chip's registers (up to 16,384 per CTA, rows whole;
  *      the load words in shared memory, at most 57,344 vertices; every weight

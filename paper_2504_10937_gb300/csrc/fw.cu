@@ -484,7 +484,7 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
         LDS_CUDA(cudaEventRecord(e0, s));
         // graphs whose slots fit the chip's registers
         bool res = false;
-        if ((g_fw_variant == 0 || g_fw_variant == 6) && (p == LDS_EXACT || p == LDS_FP32)) {
+        if (g_fw_variant == 0 || g_fw_variant == 6) {
             if (want_last) g->fw_last.alloc(std::max<int64_t>(g->m, 1), s);
             timer.start(s);
             res = fw_resident_run(g, iters, p, want_last ? g->fw_last.get() : nullptr);
@@ -496,8 +496,8 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
         bool fast = !res && !quads && g_fw_variant != 1 && run_edge_fw_oriented(g, iters, p, true, want_last, fo, timer);
         if (res) {
             LDS_CUDA(cudaEventRecord(e1, s));
-            g->pass_kernel = "fw_resident_kernel";
-            g->pass_bytes = 8 * g->m + 8 * (int64_t)nact;
+            g->pass_kernel = p == LDS_FP64 ? "fw_resident64_kernel" : "fw_resident_kernel";
+            g->pass_bytes = 8 * g->m + (p == LDS_FP64 ? 16 : 8) * (int64_t)nact;
         } else if (quads) {
             LDS_CUDA(cudaEventRecord(e1, s));
             g->pass_kernel = "fw_quad_kernel";

@@ -209,11 +209,203 @@ const void* res_kernel(int U, bool fp32) {
     }
 }
 
+// ---- Alg. 1 literally in binary64 on the same layout: one alpha per slot in a
+// register pair, alpha <- (1 - gamma) alpha + gamma alpha_hat, every operation rounded
+// on its own (with alpha_hat 0 or 1 that is one product, plus gamma where the row
+// endpoint receives), then r_x summed left to right over row x from shared memory by
+// one thread.  The binary64 pipe issues two instructions a clock and SM, so a CTA
+// takes few slots; two launches an iteration, slot pass and row sums, took 12.3 us on
+// 567 vertices with 844 edges, 4.6 us so (1.8 us of it a row of 54 additions in turn).
+constexpr int R64_UMAX = 4;
+
+struct Res64Args {
+    const int64_t* rowptr;
+    const int32_t* col;
+    const int64_t* eshift;
+    int32_t nact, N;
+    double* words;              // [2][nact padded to 2] published loads
+    int64_t *W, *R;             // [m], [nact] out
+    double* r;                  // [nact] out
+    uint8_t* last;              // [m] or null
+};
+
+template <int U, ResSync SYNC>
+__global__ void __launch_bounds__(RES_THREADS, 1) fw_resident64_kernel(const Res64Args A) {
+    extern __shared__ __align__(16) double smd[];
+    __shared__ int32_t s_row[2];
+    const int32_t nv = A.nact, nv2 = (nv + 1) & ~1;
+    double* L = smd;                                 // loads of every vertex
+    double* S = smd + nv2;                           // this CTA's alphas, in slot order
+    const int tid = threadIdx.x;
+    const int b = blockIdx.x, G = gridDim.x;
+    if (tid < 2) {
+        const int64_t want = A.rowptr[nv] * (b + tid) / G;
+        int32_t lo = 0, hi = nv;
+        while (lo < hi) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (A.rowptr[mid] < want) lo = mid + 1; else hi = mid;
+        }
+        s_row[tid] = b + tid == G ? nv : lo;
+    }
+    __syncthreads();
+    const int32_t r0 = s_row[0], r1 = s_row[1];
+    const int64_t s0 = A.rowptr[r0], s1 = A.rowptr[r1];
+    uint32_t xy[U];
+    double alpha[U];
+    uint32_t valid = 0, took = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int64_t s = s0 + (int64_t)u * RES_THREADS + tid;
+        xy[u] = 0;
+        alpha[u] = 0.5;
+        if (s < s1) {
+            int32_t lo = r0, hi = r1;                // last row with rowptr <= s
+            while (hi - lo > 1) {
+                const int32_t mid = (lo + hi) >> 1;
+                if (A.rowptr[mid] <= s) lo = mid; else hi = mid;
+            }
+            xy[u] = ((uint32_t)lo << 16) | (uint32_t)A.col[s];
+            valid |= 1u << u;
+        }
+    }
+    for (int32_t x = tid; x < nv; x += RES_THREADS) L[x] = 0.5 * (double)(A.rowptr[x + 1] - A.rowptr[x]);
+    __syncthreads();
+    for (int32_t i = 1; i <= A.N; ++i) {
+        const double gam = 2.0 / (double)(i + 2);
+        const double om = 1.0 - gam;
+        took = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if ((valid >> u) & 1u) {
+                const uint32_t x = xy[u] >> 16, y = xy[u] & 0xffffu;
+                const double rx = L[x], ry = L[y];
+                const bool recv = rx < ry || (rx == ry && x > y);
+                double a = __dmul_rn(om, alpha[u]);
+                if (recv) {
+                    a = __dadd_rn(a, gam);
+                    took |= 1u << u;
+                }
+                alpha[u] = a;
+                S[u * RES_THREADS + tid] = a;
+            }
+        __syncthreads();
+        double* out = A.words + (int64_t)(i & 1) * nv2;
+        for (int32_t x = r0 + tid; x < r1; x += RES_THREADS) {
+            int32_t q = (int32_t)(A.rowptr[x] - s0);
+            const int32_t e = (int32_t)(A.rowptr[x + 1] - s0);
+            double acc = 0.0;
+            // eight loads ahead of the chain of additions
+            for (; q + 8 <= e; q += 8) {
+                double v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = S[q + j];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc = __dadd_rn(acc, v[j]);
+            }
+            for (; q < e; ++q) acc = __dadd_rn(acc, S[q]);
+            if (SYNC == RES_BLOCK) L[x] = acc;
+            else __stcg(out + x, acc);
+        }
+        if (SYNC == RES_BLOCK) {
+            __syncthreads();
+        } else {
+            if (SYNC == RES_CLUSTER_SYNC) cg::this_cluster().sync();
+            else cg::this_grid().sync();
+            const double2* in = reinterpret_cast<const double2*>(out);
+            double2* l2 = reinterpret_cast<double2*>(L);
+#pragma unroll 4
+            for (int32_t j = tid; j < nv2 >> 1; j += RES_THREADS) l2[j] = __ldcg(in + j);
+            __syncthreads();
+        }
+    }
+    // outputs: every alpha D rounded, R = the sum of a row's, r
+    const double D = (double)((int64_t)(A.N + 1) * (A.N + 2));
+    int64_t* SI = reinterpret_cast<int64_t*>(S);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if ((valid >> u) & 1u) {
+            const uint32_t x = xy[u] >> 16, y = xy[u] & 0xffffu;
+            const int64_t w = (int64_t)(uint32_t)llrint(alpha[u] * D);
+            SI[u * RES_THREADS + tid] = w;
+            if (x < y) {
+                const int64_t e = s0 + (int64_t)u * RES_THREADS + tid + A.eshift[x];
+                A.W[e] = w;
+                if (A.last) A.last[e] = (uint8_t)((took >> u) & 1u);
+            }
+        }
+    __syncthreads();
+    for (int32_t x = r0 + tid; x < r1; x += RES_THREADS) {
+        int64_t sum = 0;
+        for (int64_t q = A.rowptr[x] - s0; q < A.rowptr[x + 1] - s0; ++q) sum += SI[q];
+        A.R[x] = sum;
+        A.r[x] = L[x];
+    }
+}
+
+template <ResSync SYNC>
+const void* res64_kernel(int U) {
+    return U == 1 ? (const void*)fw_resident64_kernel<1, SYNC>
+           : U == 2 ? (const void*)fw_resident64_kernel<2, SYNC> : (const void*)fw_resident64_kernel<4, SYNC>;
+}
+
+// launch of either form over G CTAs
+void res_launch(const void* fn, int G, ResSync sync, size_t smem, void** args, cudaStream_t s) {
+    LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RES_SMEM));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(RES_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    if (sync == RES_CLUSTER_SYNC) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = RES_CLUSTER;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = sync == RES_GRID ? 1 : 0;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    LDS_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+}
+
 }  // namespace
 
+// The binary64 form; false when the graph does not fit.
+static bool fw_resident64_run(lds_graph* g, int32_t N, uint8_t* last) {
+    const int64_t maxdeg = std::max(g->info.max_degree, 1), slots = 2 * g->m;
+    // CTAs: one up to 1,024 slots, a cluster of 8 up to 8,192, then one per 1,024 slots
+    constexpr int64_t kShare = 1024;
+    int G = slots <= kShare ? 1
+            : slots <= RES_CLUSTER * kShare ? RES_CLUSTER : (int)std::min<int64_t>(num_sms(), (slots + kShare - 1) / kShare);
+    const int64_t most = G == 1 ? slots : slots / G + maxdeg + 1;
+    if (most > (int64_t)R64_UMAX * RES_THREADS) return false;
+    int U = 1;
+    while ((int64_t)U * RES_THREADS < most) U *= 2;
+    const size_t nv2 = ((size_t)g->nact + 1) & ~(size_t)1;
+    const size_t smem = (nv2 + (size_t)U * RES_THREADS) * sizeof(double);
+    if (smem > RES_SMEM) return false;
+    cudaStream_t s = g->stream;
+    const ResSync sync = G == 1 ? RES_BLOCK : slots <= RES_CLUSTER * kShare ? RES_CLUSTER_SYNC : RES_GRID;
+    const void* fn = sync == RES_BLOCK          ? res64_kernel<RES_BLOCK>(U)
+                     : sync == RES_CLUSTER_SYNC ? res64_kernel<RES_CLUSTER_SYNC>(U) : res64_kernel<RES_GRID>(U);
+    ensure_edge_shift(g);
+    g->fw_W.alloc(g->m, s);
+    DevBuf<double> words(2 * nv2, s);
+    LDS_CUDA(cudaMemsetAsync(g->fw_R.get(), 0, g->n * sizeof(int64_t), s));
+    LDS_CUDA(cudaMemsetAsync(g->fw_r.get(), 0, g->n * sizeof(double), s));
+    Res64Args A{g->rowptr.get(), g->col.get(),  g->edge_shift.get(), g->nact, N, words.get(),
+                g->fw_W.get(),   g->fw_R.get(), g->fw_r.get(),       last};
+    void* args[] = {(void*)&A};
+    res_launch(fn, G, sync, smem, args, s);
+    return true;
+}
+
 bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last) {
-    if (p != LDS_EXACT && p != LDS_FP32) return false;
     if (N < 1 || g->m < 1 || g->nact > 65536) return false;
+    if (p == LDS_FP64) return fw_resident64_run(g, N, last);
     const bool fp32 = p == LDS_FP32;
     const int64_t maxdeg = std::max(g->info.max_degree, 1), slots = 2 * g->m;
     const unsigned __int128 D = (unsigned __int128)(N + 1) * (unsigned __int128)(N + 2);
@@ -242,7 +434,6 @@ bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last) {
     const void* fn = sync == RES_BLOCK          ? res_kernel<RES_BLOCK>(U, fp32)
                      : sync == RES_CLUSTER_SYNC ? res_kernel<RES_CLUSTER_SYNC>(U, fp32)
                                                 : res_kernel<RES_GRID>(U, fp32);
-    LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RES_SMEM));
     ensure_edge_shift(g);
     g->fw_W.alloc(g->m, s);
     const size_t nv4 = ((size_t)g->nact + 3) & ~(size_t)3;
@@ -253,24 +444,7 @@ bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last) {
     ResArgs A{g->rowptr.get(), g->col.get(),   g->edge_shift.get(), g->nact, N, words.get(),
               g->fw_W.get(),   g->fw_R.get(),  g->fw_r.get(),       last};
     void* args[] = {(void*)&A};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(G);
-    cfg.blockDim = dim3(RES_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    if (sync == RES_CLUSTER_SYNC) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = RES_CLUSTER;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    } else {
-        attr[0].id = cudaLaunchAttributeCooperative;
-        attr[0].val.cooperative = sync == RES_GRID ? 1 : 0;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    LDS_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
-    g_launches.fetch_add(1, std::memory_order_relaxed);
+    res_launch(fn, G, sync, smem, args, s);
     return true;
 }
 

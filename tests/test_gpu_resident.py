@@ -61,3 +61,22 @@ def test_resident_matches_the_pass(name, precision):
             assert got["D"] == want["D"]
             for k in ("r", "R", "W", "last"):
                 assert np.array_equal(got[k], want[k]), (N, k)
+
+
+@pytest.mark.parametrize("name", ["edge", "block_limit", "past_block", "past_cluster", "hub_row", "power_law"])
+def test_resident_binary64_matches_the_launches(name):
+    from paper_2504_10937_gb300 import lds
+    n, u, v = GRAPHS[name]()
+    with lds.Graph(n, u, v) as g:
+        for N in (1, 2, 37):
+            try:
+                lds.set_fw_variant(5)
+                want = g.fw(N, precision="fp64")
+                assert g.fw_timing()["pass_kernel"] == "fw64_slot_kernel"
+            finally:
+                lds.set_fw_variant(0)
+            got = g.fw(N, precision="fp64")
+            kernel = g.fw_timing()["pass_kernel"]
+            assert (kernel == "fw_resident64_kernel") == (name != "hub_row")
+            for k in ("r", "R", "W", "last"):
+                assert np.array_equal(got[k], want[k]), (N, k)
