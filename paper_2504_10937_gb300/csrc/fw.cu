@@ -283,6 +283,7 @@ struct EdgeFwState {
 
 static void run_edge_fw(lds_graph* g, int N, lds_precision p, EdgeFwState& st, PassTimer& timer) {
     cudaStream_t s = g->stream;
+    ensure_symmetric_view(g);
     const int64_t nslots = 2 * g->m;
     const int64_t nchunks = (nslots + 31) / 32;
     const int32_t nact = g->nact;

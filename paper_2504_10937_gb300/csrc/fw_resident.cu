@@ -215,7 +215,7 @@ const void* res_kernel(int U, bool fp32) {
 // endpoint receives), then r_x summed left to right over row x from shared memory by
 // one thread.  The binary64 pipe issues two instructions a clock and SM, so a CTA
 // takes few slots; two launches an iteration, slot pass and row sums, took 12.3 us on
-// 567 vertices with 844 edges, 4.6 us so (1.8 us of it a row of 54 additions in turn).
+// 567 vertices with 844 edges, 4.6 us so, most of it a row's 54 additions in turn.
 constexpr int R64_UMAX = 4;
 
 struct Res64Args {

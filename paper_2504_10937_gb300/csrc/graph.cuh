@@ -21,6 +21,7 @@ struct lds_graph {
     lds::DevBuf<int32_t> eu, ev;      // [m] canonical edges, internal ids, u < v
     lds::DevBuf<int64_t> rowptr;      // [nact + 1]
     lds::DevBuf<int32_t> col;         // [2m] internal ids, ascending in each row
+    // symmetric FW view (lazy)
     lds::DevBuf<int32_t> fwcol;       // [2m] col with bit 31 set on the first slot of each row
     lds::DevBuf<int32_t> chunk_row0;  // [ceil(2m / 32)] row of slot 32 g
     // [nact] (lazy): slot q of row x with col[q] > x is canonical edge q + edge_shift[x]
@@ -93,6 +94,9 @@ namespace lds {
 // buffers' stream-ordered frees then follow s.  The caller makes sure that no
 // work on the previous stream is pending.
 void set_stream(lds_graph* g, cudaStream_t s);
+
+// Builds fwcol and chunk_row0 if not present.
+void ensure_symmetric_view(lds_graph* g);
 
 // Builds edge_shift if not present.
 void ensure_edge_shift(lds_graph* g);
