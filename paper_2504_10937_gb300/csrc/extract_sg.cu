@@ -646,18 +646,18 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
     }
 }
 
-__global__ void vt_key_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt, uint64_t* key,
+__global__ void vt_key_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt, uint32_t* key,
                               uint32_t* tid) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 3 * nt; i += stride) {
         int64_t t = i / 3;
         int k = (int)(i % 3);
-        key[i] = (uint64_t)(k == 0 ? ta[t] : (k == 1 ? tb[t] : tc[t]));
+        key[i] = (uint32_t)(k == 0 ? ta[t] : (k == 1 ? tb[t] : tc[t]));
         tid[i] = (uint32_t)t;
     }
 }
 
-__global__ void vt_ptr_kernel(const uint64_t* key, int64_t k3, int32_t nact, int64_t* ptr) {
+__global__ void vt_ptr_kernel(const uint32_t* key, int64_t k3, int32_t nact, int64_t* ptr) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k3; i += stride) {
         int64_t x = (int64_t)key[i];
@@ -666,11 +666,6 @@ __global__ void vt_ptr_kernel(const uint64_t* key, int64_t k3, int32_t nact, int
         if (i == k3 - 1)
             for (int64_t r = x + 1; r <= nact; ++r) ptr[r] = k3;
     }
-}
-
-__global__ void u32_to_i32_kernel(const uint32_t* in, int64_t k, int32_t* out) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += stride) out[i] = (int32_t)in[i];
 }
 
 }  // namespace
@@ -685,12 +680,11 @@ void build_vertex_triangles(const int32_t* ta, const int32_t* tb, const int32_t*
         LDS_CUDA(cudaStreamSynchronize(s));
         return;
     }
-    DevBuf<uint64_t> key(3 * nt, s);
-    DevBuf<uint32_t> tid(3 * nt, s);
-    LDS_LAUNCH(vt_key_kernel, grid_for(3 * nt, blk), blk, 0, s, ta, tb, tc, nt, key.get(), tid.get());
-    radix_sort_u64(key.get(), tid.get(), 3 * nt, bit_length_u64((uint64_t)nact), s);
+    DevBuf<uint32_t> key(3 * nt, s);
+    uint32_t* tid = reinterpret_cast<uint32_t*>(vt_idx.get());
+    LDS_LAUNCH(vt_key_kernel, grid_for(3 * nt, blk), blk, 0, s, ta, tb, tc, nt, key.get(), tid);
+    radix_sort_u32(key.get(), tid, 3 * nt, bit_length_u64((uint64_t)nact - 1), s);
     LDS_LAUNCH(vt_ptr_kernel, grid_for(3 * nt, blk), blk, 0, s, key.get(), 3 * nt, nact, vt_ptr.get());
-    LDS_LAUNCH(u32_to_i32_kernel, grid_for(3 * nt, blk), blk, 0, s, tid.get(), 3 * nt, vt_idx.get());
     LDS_CUDA(cudaStreamSynchronize(s));
 }
 

@@ -66,7 +66,7 @@ __global__ void tv_count_kernel(const int32_t* ta, const int32_t* tb, const int3
     }
 }
 
-__global__ void tv_rank_keys_kernel(const int32_t* cnt, const int64_t* vt_ptr, int32_t nact, uint64_t* key,
+__global__ void tv_rank_keys_kernel(const int32_t* cnt, const int64_t* vt_ptr, int32_t nact, uint32_t* key,
                                     uint32_t* id) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride) {
@@ -76,14 +76,14 @@ __global__ void tv_rank_keys_kernel(const int32_t* cnt, const int64_t* vt_ptr, i
     }
 }
 
-__global__ void tv_rank_kernel(const uint64_t* key, const uint32_t* id, int32_t nact, int32_t* perm, int32_t* rank,
+__global__ void tv_rank_kernel(const uint32_t* key, const uint32_t* id, int32_t nact, int32_t* perm, int32_t* rank,
                                uint32_t* count) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nact; p += stride) {
         const int32_t x = (int32_t)id[p];
         perm[p] = x;
         rank[x] = (int32_t)p + 1;                // id 0 is padding
-        count[p] = 0xffffffffu - (uint32_t)key[p];
+        count[p] = 0xffffffffu - key[p];
     }
 }
 
@@ -349,15 +349,14 @@ static void ensure_tri_view(lds_graph* g) {
     const int32_t nact = g->nact;
     const int64_t nt = g->ntri;
     DevBuf<int32_t> rank(nact, s), cnt(g->vt_ptr.p ? 0 : nact, s);
-    DevBuf<uint64_t> key(nact, s);
-    DevBuf<uint32_t> id(nact, s);
+    DevBuf<uint32_t> key(nact, s), id(nact, s);
     if (!g->vt_ptr.p) {
         LDS_CUDA(cudaMemsetAsync(cnt.get(), 0, nact * sizeof(int32_t), s));
         LDS_LAUNCH(tv_count_kernel, grid_for(nt, blk), blk, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), nt, cnt.get());
     }
     LDS_LAUNCH(tv_rank_keys_kernel, grid_for(nact, blk), blk, 0, s, cnt.get(), g->vt_ptr.get(), nact, key.get(),
                id.get());
-    radix_sort_u64(key.get(), id.get(), nact, 32, s);
+    radix_sort_u32(key.get(), id.get(), nact, 32, s);
     g->tv_perm.alloc(nact, s);
     g->tv_count.alloc(nact, s);
     LDS_LAUNCH(tv_rank_kernel, grid_for(nact, blk), blk, 0, s, key.get(), id.get(), nact, g->tv_perm.get(), rank.get(),

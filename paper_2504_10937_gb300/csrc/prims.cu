@@ -78,9 +78,10 @@ __global__ void scan_apply_kernel(const In* in, int64_t* out, int64_t n, const i
 }
 
 // Short scans in one launch of one block, total included: a query makes hundreds of
-// them, and the tiled form takes two to six launches each (2.5 us of host time apiece).
-// 32,768 items are four rounds of 8 per thread, about what the launches would cost.
-constexpr int64_t SCAN_SHORT = 32768;
+// them, and the tiled form takes three launches each.  One block against tiles: 5.6 and
+// 14.7 us for 100 items, 11.9 and 23.6 for 8,192, 18.0 and 25.0 for 16,384, 30.3 and
+// 24.0 for 32,768.
+constexpr int64_t SCAN_SHORT = 16384;
 constexpr int SCAN_SHORT_T = 1024;
 template <class In>
 __global__ void __launch_bounds__(SCAN_SHORT_T) scan_short_kernel(const In* in, int64_t* out, int64_t n, int64_t* total) {
@@ -176,65 +177,127 @@ void exclusive_scan_i32_dev(const int32_t* in, int64_t* out, int64_t n, cudaStre
 
 namespace {
 
-constexpr int RS_THREADS = 256;
-constexpr int RS_ROUNDS = 16;                       // keys per thread per tile
-constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;     // 4096 keys per tile
+// One pass: digit counts of every tile, their scan (digit-major), and the scatter.  The
+// scatter is bound by its latencies and by the sectors it writes: a thread takes all its
+// keys in one go, a warp ranks its share by itself, and the tile is put in digit order in
+// shared memory first, so that a tile's keys of one digit (16 to 32 on average) go out as
+// one run of neighbouring lanes.  Keys per thread: as many as fit 64 registers (two
+// blocks a multiprocessor) without spills to speak of.  Measured with 8, 12 and 16:
+//   60M 64-bit keys with payload, 18 bits: 1.87, 2.22, 2.11 ms (4.46 in rounds of 256
+//   keys with three barriers each and no reordering); 32-bit keys: 1.64, 1.60, 1.48 ms;
+//   36M 64-bit keys, 40 bits: 1.90, 1.78, 1.81 ms (2.76).
+constexpr int RS_THREADS = 512;
 constexpr int RS_WARPS = RS_THREADS / 32;
+template <class Key, bool VALS>
+constexpr int RS_ROUNDS = sizeof(Key) == 4 ? 16 : VALS ? 8 : 12;
+template <class Key, bool VALS>
+constexpr int RS_TILE = RS_THREADS * RS_ROUNDS<Key, VALS>;
 
-__global__ void rs_histogram_kernel(const uint64_t* keys, int64_t n, int shift, int64_t ntiles,
-                                    int64_t* counts) {
+template <class Key, bool VALS>
+__global__ void __launch_bounds__(RS_THREADS) rs_histogram_kernel(const Key* keys, int64_t n, int shift, int64_t ntiles,
+                                                                  int32_t* counts) {
     __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
+    if (threadIdx.x < 256) h[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int j = 0; j < RS_ROUNDS; ++j) {
-        int64_t i = base + (int64_t)j * RS_THREADS + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 0xFF], 1u);
+    constexpr int ROUNDS = RS_ROUNDS<Key, VALS>, TILE = RS_TILE<Key, VALS>;
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+    if (base + TILE <= n) {
+        Key k[ROUNDS];
+#pragma unroll
+        for (int j = 0; j < ROUNDS; ++j) k[j] = keys[base + j * RS_THREADS + threadIdx.x];
+#pragma unroll
+        for (int j = 0; j < ROUNDS; ++j) atomicAdd(&h[(k[j] >> shift) & 0xFF], 1u);
+    } else {
+        for (int64_t i = base + threadIdx.x; i < n; i += RS_THREADS) atomicAdd(&h[(keys[i] >> shift) & 0xFF], 1u);
     }
     __syncthreads();
-    counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    if (threadIdx.x < 256) counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = (int32_t)h[threadIdx.x];
 }
 
-__global__ void rs_scatter_kernel(const uint64_t* keys_in, const uint32_t* vals_in, uint64_t* keys_out,
-                                  uint32_t* vals_out, int64_t n, int shift, int64_t ntiles,
-                                  const int64_t* offsets) {
-    __shared__ uint32_t s_base[256];
-    __shared__ uint32_t s_wcnt[RS_WARPS][256];
-    __shared__ int64_t s_goff[256];
-    int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    s_base[t] = 0;
-    s_goff[t] = offsets[(int64_t)t * ntiles + blockIdx.x];
+template <class Key, bool VALS>
+constexpr size_t rs_scatter_smem() {
+    return (size_t)RS_TILE<Key, VALS> * (sizeof(Key) + (VALS ? sizeof(uint32_t) : 0)) + RS_WARPS * 256 * sizeof(uint16_t);
+}
+
+template <class Key, bool VALS>
+__global__ void __launch_bounds__(RS_THREADS, 2) rs_scatter_kernel(const Key* __restrict__ keys_in,
+                                                                   const uint32_t* __restrict__ vals_in, Key* keys_out,
+                                                                   uint32_t* vals_out, int64_t n, int shift, int64_t ntiles,
+                                                                   const int64_t* offsets) {
+    constexpr int ROUNDS = RS_ROUNDS<Key, VALS>, TILE = RS_TILE<Key, VALS>;
+    extern __shared__ __align__(16) unsigned char rsm[];
+    __shared__ int64_t goff[256];
+    __shared__ uint32_t dstart[256], wsum[8];
+    Key* sk = reinterpret_cast<Key*>(rsm);
+    uint32_t* sv = reinterpret_cast<uint32_t*>(sk + TILE);
+    uint16_t* wcnt = reinterpret_cast<uint16_t*>(sv + (VALS ? TILE : 0));      // [RS_WARPS][256]
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+    const int cnt = (int)min((int64_t)TILE, n - base);
+    const int first = warp * (32 * ROUNDS) + lane;
+    Key k[ROUNDS];
 #pragma unroll
-    for (int w = 0; w < RS_WARPS; ++w) s_wcnt[w][t] = 0;
+    for (int j = 0; j < ROUNDS; ++j) k[j] = first + 32 * j < cnt ? keys_in[base + first + 32 * j] : Key(0);
+    int64_t off = 0;
+    if (t < 256) off = offsets[(int64_t)t * ntiles + blockIdx.x];
+    for (int i = t; i < RS_WARPS * 128; i += RS_THREADS) reinterpret_cast<uint32_t*>(wcnt)[i] = 0;
     __syncthreads();
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    int64_t base = (int64_t)blockIdx.x * RS_TILE;
-    for (int j = 0; j < RS_ROUNDS; ++j) {
-        int64_t i = base + (int64_t)j * RS_THREADS + t;
-        bool valid = i < n;
-        uint64_t key = valid ? keys_in[i] : 0;
-        uint32_t val = (valid && vals_in) ? vals_in[i] : 0;
-        int d = valid ? (int)((key >> shift) & 0xFF) : 256;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        int rank = __popc(peers & lt_mask);
-        if (valid && rank == 0) s_wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        if (valid) {
-            uint32_t below = 0;
-            for (int w = 0; w < warp; ++w) below += s_wcnt[w][d];
-            int64_t pos = s_goff[d] + s_base[d] + below + rank;
-            keys_out[pos] = key;
-            if (vals_out) vals_out[pos] = val;
-        }
-        __syncthreads();
-        uint32_t add = 0;
+    uint16_t* mine = wcnt + warp * 256;
+    uint32_t rk[ROUNDS / 2];                      // two ranks a word
+#pragma unroll
+    for (int j = 0; j < ROUNDS; ++j) {
+        const int d = first + 32 * j < cnt ? (int)((k[j] >> shift) & 0xFF) : 256;
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = d < 256 ? mine[d] : 0;
+        __syncwarp();
+        if (d < 256 && (peers & lt) == 0) mine[d] = (uint16_t)(before + __popc(peers));
+        __syncwarp();
+        const uint32_t r = before + __popc(peers & lt);
+        if (j & 1) rk[j / 2] |= r << 16;
+        else rk[j / 2] = r;
+    }
+    __syncthreads();
+    uint32_t run = 0, incl = 0;
+    if (t < 256) {
 #pragma unroll
         for (int w = 0; w < RS_WARPS; ++w) {
-            add += s_wcnt[w][t];
-            s_wcnt[w][t] = 0;
+            const uint32_t c = wcnt[w * 256 + t];
+            wcnt[w * 256 + t] = (uint16_t)run;
+            run += c;
         }
-        s_base[t] += add;
-        __syncthreads();
+        incl = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+    }
+    __syncthreads();
+    if (t < 256) {
+        uint32_t st = incl - run;
+        for (int w = 0; w < warp; ++w) st += wsum[w];
+        dstart[t] = st;
+        goff[t] = off - st;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < ROUNDS; ++j) {
+        if (first + 32 * j < cnt) {
+            const int d = (int)((k[j] >> shift) & 0xFF);
+            const uint32_t pos = dstart[d] + mine[d] + ((rk[j / 2] >> (16 * (j & 1))) & 0xFFFFu);
+            sk[pos] = k[j];
+            if (VALS) sv[pos] = vals_in[base + first + 32 * j];
+        }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int i = t; i < cnt; i += RS_THREADS) {
+        const Key x = sk[i];
+        const int64_t at = goff[(int)((x >> shift) & 0xFF)] + i;
+        keys_out[at] = x;
+        if (VALS) vals_out[at] = sv[i];
     }
 }
 
@@ -242,16 +305,18 @@ __global__ void rs_scatter_kernel(const uint64_t* keys_in, const uint32_t* vals_
 // payload) ping-pong in shared memory.  A warp owns a contiguous segment and ranks it
 // 32 keys at a time (lanes of equal digit by match), counting per warp and digit; one
 // scan over (digit, warp) then places every key, so each pass is stable and takes four
-// block barriers.  The tiled form takes four to six launches a pass.
+// block barriers.  The tiled form takes three to five launches a pass: 36-bit keys take
+// 34 us here and 138 us there for 4,096 of them, 57 and 148 us for 8,192, which is what
+// shared memory holds.
 constexpr int RS_SMALL = 8192;
 constexpr int RS_SMALL_T = 1024;
 constexpr int RS_SMALL_ROUNDS = RS_SMALL / RS_SMALL_T;
-template <bool VALS>
-__global__ void __launch_bounds__(RS_SMALL_T, 1) rs_small_kernel(uint64_t* keys, uint32_t* vals, int n, int passes) {
+template <class Key, bool VALS>
+__global__ void __launch_bounds__(RS_SMALL_T, 1) rs_small_kernel(Key* keys, uint32_t* vals, int n, int passes) {
     extern __shared__ __align__(16) unsigned char rsm[];
     __shared__ uint32_t dtot[256], wsum[8];
-    uint64_t* ka = reinterpret_cast<uint64_t*>(rsm);
-    uint64_t* kb = ka + n;
+    Key* ka = reinterpret_cast<Key*>(rsm);
+    Key* kb = ka + n;
     uint32_t* va = reinterpret_cast<uint32_t*>(kb + n);
     uint32_t* vb = va + (VALS ? n : 0);
     uint16_t* wcnt = reinterpret_cast<uint16_t*>(vb + (VALS ? n : 0));        // [32][256]
@@ -303,7 +368,7 @@ __global__ void __launch_bounds__(RS_SMALL_T, 1) rs_small_kernel(uint64_t* keys,
             if (r * 32 >= seg) break;
             const int i = first + r * 32 + lane;
             if (i < n) {
-                const uint64_t k = ka[i];
+                const Key k = ka[i];
                 const int d = (int)((k >> shift) & 0xFF);
                 uint32_t pos = dtot[d] + mine[d] + rk[r];
                 for (int w = 0; w < (d >> 5); ++w) pos += wsum[w];
@@ -312,7 +377,7 @@ __global__ void __launch_bounds__(RS_SMALL_T, 1) rs_small_kernel(uint64_t* keys,
             }
         }
         __syncthreads();
-        uint64_t* tk = ka;
+        Key* tk = ka;
         ka = kb;
         kb = tk;
         uint32_t* tv = va;
@@ -332,45 +397,53 @@ __global__ void gather_u32_kernel(const uint32_t* in, const uint32_t* idx, uint3
 
 }  // namespace
 
-void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s) {
+template <class Key, bool VALS>
+static void radix_sort(Key* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s) {
     if (n <= 1 || bits <= 0) return;
-    int passes = (bits + 7) / 8;
+    const int passes = (bits + 7) / 8;
     if (n <= RS_SMALL) {
-        const size_t smem = (size_t)n * (vals ? 24 : 16) + 32 * 256 * sizeof(uint16_t) + 16;
-        const size_t most = (size_t)RS_SMALL * 24 + 32 * 256 * sizeof(uint16_t) + 16;
-        if (vals) {
-            LDS_CUDA(cudaFuncSetAttribute(rs_small_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
-            LDS_LAUNCH(rs_small_kernel<true>, 1, RS_SMALL_T, smem, s, keys, vals, (int)n, passes);
-        } else {
-            LDS_CUDA(cudaFuncSetAttribute(rs_small_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
-            LDS_LAUNCH(rs_small_kernel<false>, 1, RS_SMALL_T, smem, s, keys, vals, (int)n, passes);
-        }
+        constexpr size_t per = 2 * (sizeof(Key) + (VALS ? sizeof(uint32_t) : 0)), fixed = 32 * 256 * sizeof(uint16_t);
+        LDS_CUDA(cudaFuncSetAttribute(rs_small_kernel<Key, VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(RS_SMALL * per + fixed)));
+        auto kernel = rs_small_kernel<Key, VALS>;
+        LDS_LAUNCH(kernel, 1, RS_SMALL_T, (size_t)n * per + fixed, s, keys, vals, (int)n, passes);
         return;
     }
-    int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
-    DevBuf<uint64_t> kbuf(n, s);
+    const int64_t ntiles = (n + RS_TILE<Key, VALS> - 1) / RS_TILE<Key, VALS>;
+    constexpr size_t smem = rs_scatter_smem<Key, VALS>();
+    auto histogram = rs_histogram_kernel<Key, VALS>;
+    auto scatter = rs_scatter_kernel<Key, VALS>;
+    LDS_CUDA(cudaFuncSetAttribute(scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DevBuf<Key> kbuf(n, s);
     DevBuf<uint32_t> vbuf;
-    if (vals) vbuf.alloc(n, s);
-    DevBuf<int64_t> counts(256 * ntiles, s);
-    uint64_t* kin = keys;
-    uint64_t* kout = kbuf.get();
+    if (VALS) vbuf.alloc(n, s);
+    DevBuf<int32_t> counts(256 * ntiles, s);
+    DevBuf<int64_t> offs(256 * ntiles, s);
+    Key* kin = keys;
+    Key* kout = kbuf.get();
     uint32_t* vin = vals;
-    uint32_t* vout = vals ? vbuf.get() : nullptr;
+    uint32_t* vout = VALS ? vbuf.get() : nullptr;
     for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
-        LDS_LAUNCH(rs_histogram_kernel, (unsigned)ntiles, RS_THREADS, 0, s, kin, n, shift, ntiles, counts.get());
-        LDS_CHECK_LAUNCH();
-        exclusive_scan_i64_dev(counts.get(), counts.get(), 256 * ntiles, nullptr, s);
-        LDS_LAUNCH(rs_scatter_kernel, (unsigned)ntiles, RS_THREADS, 0, s, kin, vin, kout, vout, n, shift, ntiles,
-                                                                counts.get());
-        LDS_CHECK_LAUNCH();
+        const int shift = 8 * p;
+        LDS_LAUNCH(histogram, (unsigned)ntiles, RS_THREADS, 0, s, kin, n, shift, ntiles, counts.get());
+        exclusive_scan_i32_dev(counts.get(), offs.get(), 256 * ntiles, s);
+        LDS_LAUNCH(scatter, (unsigned)ntiles, RS_THREADS, smem, s, kin, vin, kout, vout, n, shift, ntiles, offs.get());
         std::swap(kin, kout);
         std::swap(vin, vout);
     }
     if (kin != keys) {
-        LDS_CUDA(cudaMemcpyAsync(keys, kin, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-        if (vals) LDS_CUDA(cudaMemcpyAsync(vals, vin, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+        LDS_CUDA(cudaMemcpyAsync(keys, kin, n * sizeof(Key), cudaMemcpyDeviceToDevice, s));
+        if (VALS) LDS_CUDA(cudaMemcpyAsync(vals, vin, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
     }
+}
+
+void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s) {
+    if (vals) radix_sort<uint64_t, true>(keys, vals, n, bits, s);
+    else radix_sort<uint64_t, false>(keys, nullptr, n, bits, s);
+}
+
+void radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s) {
+    radix_sort<uint32_t, true>(keys, vals, n, bits, s);
 }
 
 void gather_u32(const uint32_t* in, const uint32_t* idx, uint32_t* out, int64_t n, cudaStream_t s) {

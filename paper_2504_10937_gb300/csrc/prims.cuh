@@ -23,6 +23,8 @@ void exclusive_scan_i32_dev(const int32_t* in, int64_t* out, int64_t n, cudaStre
 // with an optional uint32 payload.  keys / vals are sorted in place (a
 // temporary ping-pong buffer is allocated).  vals may be null.
 void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s);
+// 32-bit keys; vals must be given.
+void radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s);
 
 // Gathers: out[i] = in[idx[i]].
 void gather_u32(const uint32_t* in, const uint32_t* idx, uint32_t* out, int64_t n, cudaStream_t s);

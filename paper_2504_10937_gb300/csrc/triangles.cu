@@ -113,6 +113,23 @@ __global__ void tri_key_a_kernel(const int32_t* ta, const uint32_t* idx, int64_t
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntri; t += stride) key[t] = (uint64_t)ta[idx[t]];
 }
 
+__global__ void tri_pack_kernel(const int32_t* a, const int32_t* b, const int32_t* c, int64_t k, int bits, uint64_t* key) {
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < k; t += stride)
+        key[t] = ((((uint64_t)a[t] << bits) | (uint64_t)b[t]) << bits) | (uint64_t)c[t];
+}
+
+__global__ void tri_unpack_kernel(const uint64_t* key, int64_t k, int bits, int32_t* a, int32_t* b, int32_t* c) {
+    const uint64_t mask = (1ull << bits) - 1ull;
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < k; t += stride) {
+        const uint64_t x = key[t];
+        a[t] = (int32_t)(x >> (2 * bits));
+        b[t] = (int32_t)((x >> bits) & mask);
+        c[t] = (int32_t)(x & mask);
+    }
+}
+
 __global__ void permute3_kernel(const int32_t* a, const int32_t* b, const int32_t* c, const uint32_t* idx, int64_t k,
                                 int32_t* oa, int32_t* ob, int32_t* oc) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -751,17 +768,24 @@ void ensure_triangles(lds_graph* g) {
     g->tc.alloc(ntri, s);
     if (ntri) {
         DevBuf<uint64_t> key(ntri, s);
-        DevBuf<uint32_t> idx(ntri, s);
         const uint64_t nn = (uint64_t)nact;
-        LDS_LAUNCH(tri_key_bc_kernel, grid_for(ntri, blk), blk, 0, s, b.get(), c.get(), ntri, (int64_t)nn, key.get(), idx.get());
-        LDS_CHECK_LAUNCH();
-        radix_sort_u64(key.get(), idx.get(), ntri, bit_length_u64(nn * nn), s);
-        LDS_LAUNCH(tri_key_a_kernel, grid_for(ntri, blk), blk, 0, s, a.get(), idx.get(), ntri, key.get());
-        LDS_CHECK_LAUNCH();
-        radix_sort_u64(key.get(), idx.get(), ntri, bit_length_u64(nn), s);
-        LDS_LAUNCH(permute3_kernel, grid_for(ntri, blk), blk, 0, s, a.get(), b.get(), c.get(), idx.get(), ntri, g->ta.get(),
-                                                            g->tb.get(), g->tc.get());
-        LDS_CHECK_LAUNCH();
+        const int bits = bit_length_u64(nn - 1);
+        if (3 * bits <= 64) {
+            // the whole triangle is the key: no payload, one sort, no gathers
+            LDS_LAUNCH(tri_pack_kernel, grid_for(ntri, blk), blk, 0, s, a.get(), b.get(), c.get(), ntri, bits, key.get());
+            radix_sort_u64(key.get(), nullptr, ntri, 3 * bits, s);
+            LDS_LAUNCH(tri_unpack_kernel, grid_for(ntri, blk), blk, 0, s, key.get(), ntri, bits, g->ta.get(), g->tb.get(),
+                       g->tc.get());
+        } else {
+            DevBuf<uint32_t> idx(ntri, s);
+            LDS_LAUNCH(tri_key_bc_kernel, grid_for(ntri, blk), blk, 0, s, b.get(), c.get(), ntri, (int64_t)nn, key.get(),
+                       idx.get());
+            radix_sort_u64(key.get(), idx.get(), ntri, bit_length_u64(nn * nn), s);
+            LDS_LAUNCH(tri_key_a_kernel, grid_for(ntri, blk), blk, 0, s, a.get(), idx.get(), ntri, key.get());
+            radix_sort_u64(key.get(), idx.get(), ntri, bit_length_u64(nn), s);
+            LDS_LAUNCH(permute3_kernel, grid_for(ntri, blk), blk, 0, s, a.get(), b.get(), c.get(), idx.get(), ntri,
+                       g->ta.get(), g->tb.get(), g->tc.get());
+        }
     }
     LDS_CUDA(cudaStreamSynchronize(s));
     g->ntri = ntri;

@@ -52,7 +52,7 @@ def test_sort_sizes(lds, n, pairs):
     _check(lds, n, a, b, fw=pairs <= 513)
 
 
-@pytest.mark.parametrize("n", [1, 8191, 8192, 8193, 32767, 32768, 32769, 3_000_001])
+@pytest.mark.parametrize("n", [1, 8191, 8192, 8193, 16383, 16384, 16385, 3_000_001])
 def test_scan_sizes_and_gaps(lds, n):
     rng = np.random.default_rng(n)
     ids = np.unique(np.concatenate([[0, n - 1], rng.integers(0, n, 9)]))
@@ -61,8 +61,8 @@ def test_scan_sizes_and_gaps(lds, n):
 
 
 def test_flag_word_scan_sizes(lds):
-    # 32 flags a word: 32,768 words and one more
-    for pairs in (524_287, 524_288, 524_289):
+    # 32 flags a word: 16,384 words and one more
+    for pairs in (262_143, 262_144, 262_145):
         rng = np.random.default_rng(pairs)
         _check(lds, 100_000, rng.integers(0, 100_000, pairs), rng.integers(0, 100_000, pairs))
 
