@@ -81,9 +81,16 @@ __global__ void sg_hist_edges_kernel(const int32_t* eu, const int32_t* ev, int64
 
 __global__ void sg_hist_tris_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt,
                                     const int32_t* pos, int32_t* h) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride)
-        atomicAdd(h + max(pos[ta[t]], max(pos[tb[t]], pos[tc[t]])), 1);
+    // neighbouring triangles share vertices, and on a skewed graph most maxima are a few
+    // positions: one addition per position and warp
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; t0 < nt; t0 += stride) {
+        const int64_t t = t0 + lane;
+        const int32_t p = t < nt ? max(pos[ta[t]], max(pos[tb[t]], pos[tc[t]])) : -1;
+        const unsigned peers = __match_any_sync(0xffffffffu, p);
+        if (p >= 0 && lane == __ffs(peers) - 1) atomicAdd(h + p, __popc(peers));
+    }
 }
 
 constexpr int CUT_THREADS = 256;

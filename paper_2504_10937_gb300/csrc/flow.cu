@@ -378,6 +378,86 @@ __global__ void hyper_pos_kernel(const int64_t* pptr, const int32_t* pidx, int32
     }
 }
 
+// The same counts and positions where few vertices take many patterns: a block counts
+// its range of patterns in shared memory, takes one run of every vertex's list from the
+// cursor, and numbers its slots within the runs, one shared addition per vertex and warp.
+// With global counters 22 million triangles over 988 vertices took 6.1 ms to count and
+// 6.4 ms to place, all on the same few addresses.
+constexpr int HP_THREADS = 512;
+constexpr int HP_MAX_NV = 8192;                // 32 KB of counters a block
+__global__ void __launch_bounds__(HP_THREADS) hyper_count_runs_kernel(const int64_t* pptr, const int32_t* pidx, int32_t np,
+                                                                      const int64_t* f, int32_t nv, int64_t per,
+                                                                      int32_t* deg, ull* in, int32_t* wide, int32_t* runs) {
+    extern __shared__ int32_t hcount[];
+    for (int32_t v = threadIdx.x; v < nv; v += HP_THREADS) hcount[v] = 0;
+    __syncthreads();
+    const int64_t j0 = blockIdx.x * per, j1 = min((int64_t)np, j0 + per);
+    for (int64_t j = j0 + threadIdx.x; j < j1; j += HP_THREADS) {
+        const int64_t b = pptr[j], e = pptr[j + 1], len = e - b;
+        if (len > 3) {
+            atomicOr(wide, 1);
+            continue;
+        }
+        if (len == 3 && !(__ldcg(wide) & 2)) atomicOr(wide, 2);
+        if (len == 1) atomicAdd(in + pidx[b], (ull)f[b]);
+        else
+            for (int64_t k = b; k < e; ++k) atomicAdd(hcount + pidx[k], 1);
+    }
+    __syncthreads();
+    for (int32_t v = threadIdx.x; v < nv; v += HP_THREADS) {
+        const int32_t c = hcount[v];
+        runs[(int64_t)blockIdx.x * nv + v] = c;
+        if (c) atomicAdd(deg + v, c);
+    }
+}
+
+__global__ void __launch_bounds__(HP_THREADS) hyper_place_runs_kernel(const int64_t* pptr, const int32_t* pidx, int32_t np,
+                                                                      int32_t nv, int64_t per, const int64_t* vptr,
+                                                                      int32_t* cursor, const int32_t* runs, int32_t* pos) {
+    extern __shared__ int32_t hcount[];
+    const int lane = threadIdx.x & 31;
+    for (int32_t v = threadIdx.x; v < nv; v += HP_THREADS) {
+        const int32_t c = runs[(int64_t)blockIdx.x * nv + v];
+        hcount[v] = c ? (int32_t)vptr[v] + atomicAdd(cursor + v, c) : 0;
+    }
+    __syncthreads();
+    const int64_t j0 = blockIdx.x * per, j1 = min((int64_t)np, j0 + per);
+    for (int64_t jw = j0 + threadIdx.x - lane; jw < j1; jw += HP_THREADS) {
+        const int64_t j = jw + lane;
+        int64_t b = 0;
+        int len = 0;
+        if (j < j1) {
+            b = pptr[j];
+            len = (int)(pptr[j + 1] - b);
+        }
+        if (len < 2 || len > 3) len = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int32_t x = k < len ? pidx[b + k] : -1;
+            const unsigned peers = __match_any_sync(0xffffffffu, x);
+            const int lead = __ffs(peers) - 1;
+            int32_t at = 0;
+            if (x >= 0 && lane == lead) at = atomicAdd(hcount + x, __popc(peers));
+            at = __shfl_sync(0xffffffffu, at, lead);
+            if (x >= 0) pos[b + k] = at + __popc(peers & ((1u << lane) - 1u));
+        }
+    }
+}
+
+// in[v] += flow over v's incidences; `parts` warps a vertex
+__global__ void hyper_in_kernel(HNet net, int32_t parts, ull* in) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < (int64_t)net.nv * parts; w += nwarps) {
+        const int32_t v = (int32_t)(w / parts), part = (int32_t)(w % parts);
+        const int64_t e = net.vptr[v + 1];
+        ull sum = 0;
+        for (int64_t i = net.vptr[v] + part * 32 + lane; i < e; i += 32 * (int64_t)parts) sum += (ull)net.f[i];
+        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0 && sum) atomicAdd(in + v, sum);
+    }
+}
+
 __global__ void hyper_fill_kernel(const int64_t* pptr, const int32_t* pidx, int32_t np, const int64_t* fslot,
                                   const int32_t* pos, HNet net) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -679,7 +759,16 @@ static int64_t hyper_max_flow(const int64_t* pptr, const int32_t* pidx, int32_t 
     LDS_CUDA(cudaMemsetAsync(wide.get(), 0, sizeof(int32_t), s));
     LDS_CUDA(cudaMemsetAsync(in.get(), 0, nvp * sizeof(ull), s));
     LDS_CUDA(cudaMemsetAsync(ctrl.get(), 0, HC_WORDS * sizeof(ull), s));
-    if (np)
+    // counters per block: at least as many patterns a block as it has counters to flush
+    const int64_t blocks = std::min<int64_t>(2 * num_sms(), np / std::max(nv, 1024));
+    const bool by_runs = nv > 0 && nv <= HP_MAX_NV && blocks >= 2;
+    const int64_t per = by_runs ? (np + blocks - 1) / blocks : 0;
+    const size_t hsmem = (size_t)nv * sizeof(int32_t);
+    DevBuf<int32_t> runs(by_runs ? blocks * nv : 0, s);
+    if (by_runs)
+        LDS_LAUNCH(hyper_count_runs_kernel, (unsigned)blocks, HP_THREADS, hsmem, s, pptr, pidx, np, fslot, nv, per, deg.get(),
+                   in.get(), wide.get(), runs.get());
+    else if (np)
         LDS_LAUNCH(hyper_degree_kernel, grid_for(np, FB), FB, 0, s, pptr, pidx, np, fslot, deg.get(), in.get(),
                    wide.get());
     DevBuf<int64_t> vptr(nvp + 1, s);
@@ -707,8 +796,16 @@ static int64_t hyper_max_flow(const int64_t* pptr, const int32_t* pidx, int32_t 
                    chunk.get());
     }
     if (np) {
-        LDS_LAUNCH(hyper_pos_kernel, grid_for(np, FB), FB, 0, s, pptr, pidx, np, vptr.get(), cursor.get(), pos.get());
+        if (by_runs)
+            LDS_LAUNCH(hyper_place_runs_kernel, (unsigned)blocks, HP_THREADS, hsmem, s, pptr, pidx, np, nv, per, vptr.get(),
+                       cursor.get(), runs.get(), pos.get());
+        else
+            LDS_LAUNCH(hyper_pos_kernel, grid_for(np, FB), FB, 0, s, pptr, pidx, np, vptr.get(), cursor.get(), pos.get());
         LDS_LAUNCH(hyper_fill_kernel, grid_for(np, FB), FB, 0, s, pptr, pidx, np, fslot, pos.get(), net);
+        if (by_runs) {
+            const int32_t parts = (int32_t)std::max(1, 16384 / nv);
+            LDS_LAUNCH(hyper_in_kernel, grid_for((int64_t)nv * parts * 32, FB), FB, 0, s, net, parts, in.get());
+        }
     }
     if (nv) LDS_LAUNCH(hyper_init_kernel, grid_for(nv, FB), FB, 0, s, net, in.get(), pK, ctrl.get() + HC_FLOW);
     if (nv) {

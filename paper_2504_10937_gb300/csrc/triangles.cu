@@ -32,41 +32,51 @@ __device__ __forceinline__ bool precedes(int32_t dx, int32_t x, int32_t dy, int3
     return dx < dy || (dx == dy && x < y);
 }
 
+// One warp per row, ballots keeping the row's order: a thread per row left the hubs' rows
+// (10^4 neighbours, each with two dependent loads) to one lane; 7.1 ms for the two passes
+// over 3.6 million edges of an R-MAT graph.
 __global__ void orient_count_kernel(const int64_t* rowptr, const int32_t* col, int32_t nact, int32_t* outdeg) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride) {
-        int64_t b = rowptr[x], e = rowptr[x + 1];
-        int32_t dx = (int32_t)(e - b);
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < nact; x += nwarps) {
+        const int64_t b = rowptr[x], e = rowptr[x + 1];
+        const int32_t dx = (int32_t)(e - b);
         int32_t c = 0;
-        for (int64_t s = b; s < e; ++s) {
-            int32_t y = col[s];
-            int32_t dy = (int32_t)(rowptr[y + 1] - rowptr[y]);
-            c += precedes(dx, (int32_t)x, dy, y);
+        for (int64_t s = b + lane; s < e; s += 32) {
+            const int32_t y = col[s];
+            c += precedes(dx, (int32_t)x, (int32_t)(rowptr[y + 1] - rowptr[y]), y);
         }
-        outdeg[x] = c;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) outdeg[x] = c;
     }
 }
 
+// oriented neighbours and the source vertex of every oriented slot
 __global__ void orient_fill_kernel(const int64_t* rowptr, const int32_t* col, int32_t nact, const int64_t* optr,
-                                   int32_t* ocol) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride) {
-        int64_t b = rowptr[x], e = rowptr[x + 1];
-        int32_t dx = (int32_t)(e - b);
+                                   int32_t* ocol, int32_t* osrc) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < nact; x += nwarps) {
+        const int64_t b = rowptr[x], e = rowptr[x + 1];
+        const int32_t dx = (int32_t)(e - b);
         int64_t o = optr[x];
-        for (int64_t s = b; s < e; ++s) {
-            int32_t y = col[s];
-            int32_t dy = (int32_t)(rowptr[y + 1] - rowptr[y]);
-            if (precedes(dx, (int32_t)x, dy, y)) ocol[o++] = y;
+        for (int64_t s0 = b; s0 < e; s0 += 32) {
+            const int64_t s = s0 + lane;
+            int32_t y = 0;
+            bool take = false;
+            if (s < e) {
+                y = col[s];
+                take = precedes(dx, (int32_t)x, (int32_t)(rowptr[y + 1] - rowptr[y]), y);
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            if (take) {
+                const int64_t at = o + __popc(m & ((1u << lane) - 1u));
+                ocol[at] = y;
+                osrc[at] = (int32_t)x;
+            }
+            o += __popc(m);
         }
     }
-}
-
-// source vertex of every oriented slot
-__global__ void oriented_src_kernel(const int64_t* optr, int32_t nact, int32_t* osrc) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nact; x += stride)
-        for (int64_t s = optr[x], e = optr[x + 1]; s < e; ++s) osrc[s] = (int32_t)x;
 }
 
 template <bool WRITE>
@@ -740,14 +750,14 @@ void ensure_triangles(lds_graph* g) {
     }
     DevBuf<int32_t> outdeg(nact + 1, s);
     LDS_CUDA(cudaMemsetAsync(outdeg.get(), 0, (nact + 1) * sizeof(int32_t), s));
-    LDS_LAUNCH(orient_count_kernel, grid_for(nact, blk), blk, 0, s, g->rowptr.get(), g->col.get(), nact, outdeg.get());
+    LDS_LAUNCH(orient_count_kernel, grid_for((int64_t)nact * 32, blk), blk, 0, s, g->rowptr.get(), g->col.get(), nact, outdeg.get());
     LDS_CHECK_LAUNCH();
     DevBuf<int64_t> optr(nact + 1, s);
     int64_t nos = exclusive_scan_i32_to_i64(outdeg.get(), optr.get(), nact + 1, s);
     LDS_REQUIRE(nos == g->m, LDS_ECUDA, "triangle listing: orientation lost edges (internal error)");
     DevBuf<int32_t> ocol(nos, s), osrc(nos, s);
-    LDS_LAUNCH(orient_fill_kernel, grid_for(nact, blk), blk, 0, s, g->rowptr.get(), g->col.get(), nact, optr.get(), ocol.get());
-    LDS_LAUNCH(oriented_src_kernel, grid_for(nact, blk), blk, 0, s, optr.get(), nact, osrc.get());
+    LDS_LAUNCH(orient_fill_kernel, grid_for((int64_t)nact * 32, blk), blk, 0, s, g->rowptr.get(), g->col.get(), nact,
+               optr.get(), ocol.get(), osrc.get());
     LDS_CHECK_LAUNCH();
     DevBuf<int64_t> cnt(nos, s), off(nos, s);
     LDS_LAUNCH(tri_intersect_kernel<false>, grid_for(nos, blk), blk, 0, s, optr.get(), ocol.get(), osrc.get(), nos, cnt.get(),
