@@ -301,42 +301,66 @@ __device__ __forceinline__ uint32_t weighted(uint32_t w, uint32_t first) {
            8 * __popc(w & 0xff00ff00u) + 16 * __popc(w & 0xffff0000u);
 }
 
-// A block takes 8 chunks (32 words of each plane), 32 iterations at a time: the words
-// of 32 iterations are transposed in the warp, so a lane holds one entry's 32 choices
-// and adds their weights by six popcounts, where a loop over the planes took four
-// instructions per choice (1M-vertex power law, 500 planes: 1.8 ms that way).
-constexpr int FQ_CHUNKS = 8;
+// A warp takes two chunks (one 32-byte sector of each plane) and a lane one of 32
+// iterations, the next 32 on their way: each word is transposed in the warp, so a lane
+// holds one entry's 32 choices and adds their weights by six popcounts, and a chunk's
+// entries are written whole.  No barrier and no shared memory: a block of 32 warps that
+// exchanged the words through it waited for memory and for itself in turn (22 million
+// triangles, planes of 2 GB: 1.63 ms, 1.31 so; the popcounts and shuffles bound it now,
+// the planes' bytes would take 0.3 ms).
+constexpr int FQ_THREADS = 256;
 template <int P>
-__global__ void __launch_bounds__(1024) fold_quads_kernel(const uint32_t* __restrict__ planes, int nplanes,
-                                                          int64_t nchunks, int64_t i_first, uint32_t mult, uint32_t* W0,
-                                                          uint32_t* W1) {
-    __shared__ uint32_t tile[P][32][33];
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const int64_t words = 4 * nchunks;
-    for (int64_t c0 = (int64_t)blockIdx.x * FQ_CHUNKS; c0 < nchunks; c0 += (int64_t)gridDim.x * FQ_CHUNKS) {
-        uint32_t acc[P];
+__global__ void __launch_bounds__(FQ_THREADS) fold_quads_kernel(const uint4* __restrict__ planes, int nplanes,
+                                                                int64_t nchunks, int64_t i_first, uint32_t mult,
+                                                                uint32_t* W0, uint32_t* W1) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t c0 = 2 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); c0 < nchunks; c0 += 2 * nwarps) {
+        const bool two = c0 + 1 < nchunks;
+        uint32_t acc[P][8];
+        uint4 cur[P][2], nxt[P][2];
+        auto fetch = [&](int k0, uint4 (&to)[P][2]) {
+            const int64_t k = k0 + lane;
 #pragma unroll
-        for (int p = 0; p < P; ++p) acc[p] = 0;
-        const int64_t at = 4 * c0 + lane;
+            for (int p = 0; p < P; ++p) {
+                const uint4* at = planes + (P * k + p) * nchunks + c0;
+                to[p][0] = k < nplanes ? __ldcs(at) : make_uint4(0, 0, 0, 0);
+                to[p][1] = k < nplanes && two ? __ldcs(at + 1) : make_uint4(0, 0, 0, 0);
+            }
+        };
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[p][j] = 0;
+        fetch(0, cur);
         for (int k0 = 0; k0 < nplanes; k0 += 32) {
-            const int k = k0 + w;
-            const bool in = k < nplanes && at < words;
-#pragma unroll
-            for (int p = 0; p < P; ++p) tile[p][w][lane] = in ? __ldcs(planes + ((int64_t)P * k + p) * words + at) : 0u;
-            __syncthreads();
-            // warp w takes word w: row l of the matrix is iteration l
+            fetch(k0 + 32, nxt);
+            const uint32_t first = (uint32_t)(i_first + k0 + 1);
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                acc[p] += mult * weighted(transpose32(tile[p][lane][w], lane), (uint32_t)(i_first + k0 + 1));
-            __syncthreads();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    acc[p][4 * h] += weighted(transpose32(cur[p][h].x, lane), first);
+                    acc[p][4 * h + 1] += weighted(transpose32(cur[p][h].y, lane), first);
+                    acc[p][4 * h + 2] += weighted(transpose32(cur[p][h].z, lane), first);
+                    acc[p][4 * h + 3] += weighted(transpose32(cur[p][h].w, lane), first);
+                    cur[p][h] = nxt[p][h];
+                }
         }
-        // word w is word (w & 3) of chunk c0 + (w >> 2)
-        const int64_t ch = c0 + (w >> 2);
-        if (ch < nchunks) {
-            const int64_t item = ch * 128 + 4 * lane + (w & 3);
-            W0[item] += acc[0];
-            if (P == 2) W1[item] += acc[P - 1];
-        }
+        // entry 4 * lane + j of a chunk is bit `lane` of its word j
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h && !two) continue;
+                uint4* at = reinterpret_cast<uint4*>((p ? W1 : W0) + (c0 + h) * 128) + lane;
+                uint4 v = *at;
+                v.x += mult * acc[p][4 * h];
+                v.y += mult * acc[p][4 * h + 1];
+                v.z += mult * acc[p][4 * h + 2];
+                v.w += mult * acc[p][4 * h + 3];
+                *at = v;
+            }
     }
 }
 
@@ -345,12 +369,10 @@ __global__ void __launch_bounds__(1024) fold_quads_kernel(const uint32_t* __rest
 void fold_quads(const uint32_t* planes, int nplanes, int64_t nchunks, int64_t i_first, uint32_t mult, uint32_t* W0,
                 uint32_t* W1, cudaStream_t s) {
     if (nplanes <= 0 || nchunks <= 0) return;
-    const unsigned grid =
-        (unsigned)std::min<int64_t>((nchunks + FQ_CHUNKS - 1) / FQ_CHUNKS, (int64_t)num_sms() * 16);
-    if (W1)
-        LDS_LAUNCH(fold_quads_kernel<2>, grid, 1024, 0, s, planes, nplanes, nchunks, i_first, mult, W0, W1);
-    else
-        LDS_LAUNCH(fold_quads_kernel<1>, grid, 1024, 0, s, planes, nplanes, nchunks, i_first, mult, W0, W1);
+    const uint4* p4 = reinterpret_cast<const uint4*>(planes);
+    const unsigned grid = grid_for((nchunks + 1) / 2 * 32, FQ_THREADS);
+    if (W1) LDS_LAUNCH(fold_quads_kernel<2>, grid, FQ_THREADS, 0, s, p4, nplanes, nchunks, i_first, mult, W0, W1);
+    else LDS_LAUNCH(fold_quads_kernel<1>, grid, FQ_THREADS, 0, s, p4, nplanes, nchunks, i_first, mult, W0, W1);
 }
 
 static void ensure_quad_view(lds_graph* g) {
