@@ -210,6 +210,39 @@ __global__ void tri_item_count_kernel(const int32_t* list, int32_t k, const int6
     }
 }
 
+// Triangle by triangle, where the members' lists together are longer than T: bit t of
+// words is set when all of t's members are in; cnt: set bits per word
+__global__ void tri_in_words_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt,
+                                    const uint8_t* in, uint32_t* words, int32_t* cnt) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5, nw = (nt + 31) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw; w += nwarps) {
+        const int64_t t = (w << 5) + lane;
+        const unsigned b = __ballot_sync(0xffffffffu, t < nt && in[ta[t]] && in[tb[t]] && in[tc[t]]);
+        if (lane == 0) {
+            words[w] = b;
+            cnt[w] = __popc(b);
+        }
+    }
+}
+
+__global__ void tri_in_fill_kernel(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt,
+                                   const uint32_t* words, const int64_t* base, const int32_t* local, int32_t* pidx,
+                                   const int64_t* W, int64_t* share) {
+    int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride) {
+        const uint32_t f = words[t >> 5];
+        const int l = (int)(t & 31);
+        if (!((f >> l) & 1u)) continue;
+        const int64_t at = 3 * (base[t >> 5] + __popc(f & ((1u << l) - 1u)));
+        pidx[at] = local[ta[t]];
+        pidx[at + 1] = local[tb[t]];
+        pidx[at + 2] = local[tc[t]];
+        if (share)
+            for (int j = 0; j < 3; ++j) share[at + j] = W[3 * t + j];
+    }
+}
+
 // per taking item: its pattern's start (slot offset) and members, with the
 // Frank-Wolfe split of each member when share is given
 __global__ void tri_item_fill_kernel(const int32_t* list, int32_t k, const int64_t* ioff, int64_t nitems,
@@ -525,6 +558,29 @@ static int64_t build_patterns(lds_graph* g, bool tri, const int32_t* list, int32
         DevBuf<int64_t> ioff;
         if (k) LDS_LAUNCH(tri_inc_count_kernel, grid_for(k, VB), VB, 0, s, list, k, nact, g->vt_ptr.get(), cnt.get());
         const int64_t nitems = scan_counts(cnt.get(), k, ioff, s);
+        if (all_in && nitems >= g->ntri && g->ntri > 0) {
+            // every triangle once, in order, against each member's list with a search for the
+            // member per entry: 22 million triangles of 988 vertices, 6.7 ms that way
+            const int64_t nt = g->ntri, nw = (nt + 31) / 32;
+            DevBuf<uint32_t> words(nw, s);
+            DevBuf<int32_t> wcnt(nw, s);
+            DevBuf<int64_t> base(nw, s);
+            LDS_LAUNCH(tri_in_words_kernel, grid_for(nt, VB), VB, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), nt,
+                       sc.in.get(), words.get(), wcnt.get());
+            const int64_t np = exclusive_scan_i32_to_i64(wcnt.get(), base.get(), nw, s);
+            pptr.alloc(np + 1, s);
+            pidx.alloc(std::max<int64_t>(3 * np, 1), s);
+            if (warm) share->alloc(std::max<int64_t>(3 * np, 1), s);
+            LDS_LAUNCH(uniform_pat_ptr_kernel, grid_for(np + 1, VB), VB, 0, s, np, 3, pptr.get());
+            if (np)
+                LDS_LAUNCH(tri_in_fill_kernel, grid_for(nt, VB), VB, 0, s, g->ta.get(), g->tb.get(), g->tc.get(), nt,
+                           words.get(), base.get(), sc.local.get(), pidx.get(),
+                           warm ? (const int64_t*)g->fw_W.get() : (const int64_t*)nullptr,
+                           warm ? share->get() : (int64_t*)nullptr);
+            LDS_CUDA(cudaStreamSynchronize(s));
+            if (n_main) *n_main = np;
+            return np;
+        }
         DevBuf<int32_t> take(nitems + 1, s), plen(all_in ? 0 : nitems + 1, s);
         if (nitems)
             LDS_LAUNCH(tri_item_count_kernel, grid_for(nitems, VB), VB, 0, s, list, k, ioff.get(), nitems,
