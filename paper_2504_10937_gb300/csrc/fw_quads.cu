@@ -305,7 +305,7 @@ __device__ __forceinline__ uint32_t weighted(uint32_t w, uint32_t first) {
 // iterations, the next 32 on their way: each word is transposed in the warp, so a lane
 // holds one entry's 32 choices and adds their weights by six popcounts, and a chunk's
 // entries are written whole.  No barrier and no shared memory: a block of 32 warps that
-// exchanged the words through it waited for memory and for itself in turn (22 million
+// exchanged the words through it waited for memory and for itself in turn (84.6 million
 // triangles, planes of 2 GB: 1.63 ms, 1.31 so; the popcounts and shuffles bound it now,
 // the planes' bytes would take 0.3 ms).
 constexpr int FQ_THREADS = 256;
