@@ -680,9 +680,9 @@ __global__ void vt_ptr_kernel(const uint32_t* key, int64_t k3, int32_t nact, int
 void build_vertex_triangles(const int32_t* ta, const int32_t* tb, const int32_t* tc, int64_t nt, int32_t nact,
                             DevBuf<int64_t>& vt_ptr, DevBuf<int32_t>& vt_idx, cudaStream_t s) {
     const int blk = 256;
-    vt_ptr.alloc(nact + 1, s);
     vt_idx.alloc(std::max<int64_t>(3 * nt, 1), s);
     if (nt == 0) {
+        vt_ptr.alloc(nact + 1, s);
         LDS_CUDA(cudaMemsetAsync(vt_ptr.get(), 0, (nact + 1) * sizeof(int64_t), s));
         LDS_CUDA(cudaStreamSynchronize(s));
         return;
@@ -691,6 +691,7 @@ void build_vertex_triangles(const int32_t* ta, const int32_t* tb, const int32_t*
     uint32_t* tid = reinterpret_cast<uint32_t*>(vt_idx.get());
     LDS_LAUNCH(vt_key_kernel, grid_for(3 * nt, blk), blk, 0, s, ta, tb, tc, nt, key.get(), tid);
     radix_sort_u32(key.get(), tid, 3 * nt, bit_length_u64((uint64_t)nact - 1), s);
+    vt_ptr.alloc(nact + 1, s);       // last: its presence says that the index is whole
     LDS_LAUNCH(vt_ptr_kernel, grid_for(3 * nt, blk), blk, 0, s, key.get(), 3 * nt, nact, vt_ptr.get());
     LDS_CUDA(cudaStreamSynchronize(s));
 }
