@@ -45,6 +45,7 @@ constexpr int EQ_THREADS = 1024;
 constexpr int EQ_CHUNK = 32;                     // quads of a warp step
 constexpr int32_t EQ_HOT = 38144;                // hot ids: 4 B of load and 2 B of count each
 constexpr size_t EQ_SMEM = (size_t)EQ_HOT * 6;
+constexpr int32_t EQ_HOT_LEAST = 4096;
 
 __device__ __forceinline__ unsigned lanes_le(int lane) { return lane == 31 ? FULL : (2u << lane) - 1u; }
 
@@ -436,8 +437,17 @@ bool run_edge_fw_quads(lds_graph* g, int N, lds_precision p, bool want_last, Pas
     LDS_CUDA(cudaMemsetAsync(W.get(), 0, 128 * nchunks * sizeof(uint32_t), s));
     const void* fn = fp32 ? (const void*)fw_quad_kernel<float> : (const void*)fw_quad_kernel<uint32_t>;
     LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)EQ_SMEM));
-    const int32_t nhot = (int32_t)std::min<int64_t>((int64_t)nact + 1, EQ_HOT);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms(), (nchunks + 31) / 32));
+    // Hot ids: twice the entries of a block's share, so that staging and flushing them stays
+    // in proportion to the pass (both take every block of every iteration).  Staged whole,
+    // graphs of 55,000 to 200,000 vertices spent more on it than on their edges: 58,000
+    // vertices with 291k edges, exact, 11.3 us an iteration with 38,144 ids, 8.9 with 8,192,
+    // 8.6 with 4,096, 9.0 with none (9.1 by this rule); 400,000 with 817k edges 14.8, 13.2,
+    // 12.8, 14.8, and 12.5 with 16,384 (13.1 by this rule).  Past 2.9M entries or so every
+    // id that fits is staged.
+    const int64_t share = 4 * EQ_CHUNK * nchunks / grid;
+    const int32_t nhot =
+        (int32_t)std::min<int64_t>((int64_t)nact + 1, std::min<int64_t>(EQ_HOT, std::max<int64_t>(EQ_HOT_LEAST, 2 * share)));
     int stored = 0;
     for (int i = 1; i <= N; i += stored) {
         stored = std::min(K, N - i + 1);
