@@ -45,6 +45,7 @@ constexpr int TQ_THREADS = 1024;
 constexpr int TQ_CHUNK = 32;                     // quads of a warp step
 constexpr size_t TQ_SMEM = 224 * 1024;
 constexpr int32_t TQ_HOT = (int32_t)(TQ_SMEM / 8) - 8;     // hot ids with 4-byte loads: 4 B and a 4 B counter
+constexpr int64_t TQ_HOT_LEAST = 4096;
 
 __device__ __forceinline__ unsigned lanes_le(int lane) { return lane == 31 ? FULL : (2u << lane) - 1u; }
 
@@ -423,14 +424,27 @@ void run_tri_fw(lds_graph* g, int N, lds_precision p, bool want_last, PassTimer&
     const void* fn = fp32 ? (const void*)fw_tri_quad_kernel<float> : (const void*)fw_tri_quad_kernel<int64_t>;
     LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TQ_SMEM));
     const size_t lsize = fp32 ? sizeof(float) : sizeof(int64_t);
-    const int32_t nhot =
-        (int32_t)std::min<int64_t>((int64_t)nact + 1, fp32 ? (int64_t)TQ_HOT : (int64_t)((TQ_SMEM - 32) / (lsize + 4)));
+    // Two chunks a warp at least: a block's staging and flush of the hot vertices is shared by
+    // its passes over them.  And a vertex a thread where there are blocks for it: few
+    // triangles on many vertices left the update to a few blocks (10,000 triangles on 30,000
+    // vertices: five).
+    const int grid = (int)std::max<int64_t>(
+        1, std::min<int64_t>(num_sms(), std::max<int64_t>((nchunks + 63) / 64, (nact + TQ_THREADS - 1) / TQ_THREADS)));
+    // Hot ids: twice the entries of a block's share, as in the edge pass; binary32 stages
+    // all of them when that is within an eighth of all, for the hot part's own form (144k
+    // triangles on 17,000 vertices: 8.1 us an iteration so, 8.6 without).  Microseconds an
+    // iteration, exact / binary32, of every id that fits in every block on the smaller grid,
+    // and so: 216k triangles on 100,000 vertices 15.4 / 16.4, 9.3 / 9.3; 10,000 on 30,000
+    // 13.6 / 13.7, 6.6 / 6.8; 246k on 167,000 12.4 / 11.7, 7.8 / 7.0.  From 270,000 quads or
+    // so every id that fits is staged.
+    const int64_t fit = fp32 ? (int64_t)TQ_HOT : (int64_t)((TQ_SMEM - 32) / (lsize + 4));
+    const int64_t every = std::min<int64_t>((int64_t)nact + 1, TQ_HOT);          // ids of the hot part
+    int64_t hot = std::max<int64_t>(TQ_HOT_LEAST, 2 * (4 * TQ_CHUNK * nchunks / grid));
+    if (fp32 && hot + hot / 8 >= every) hot = std::max(hot, every);
+    const int32_t nhot = (int32_t)std::min(std::min<int64_t>((int64_t)nact + 1, fit), hot);
     const size_t smem = (((size_t)nhot * lsize + 15) & ~(size_t)15) + (size_t)nhot * 4;
-    // 64-bit loads stage fewer ids: unless that is all of them, every chunk takes the general form
-    const int64_t hchunks = fp32 || nhot == nact + 1 ? g->tv_hchunks : 0;
-    // two chunks a warp at least: a block's staging and flush of the hot vertices is
-    // shared by its passes over them
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms(), (nchunks + 63) / 64));
+    // the hot part's own form needs all of its ids staged; else every chunk takes the general one
+    const int64_t hchunks = nhot >= every ? g->tv_hchunks : 0;
     int stored = 0;
     for (int i = 1; i <= N; i += stored) {
         stored = std::min(K, N - i + 1);
