@@ -212,22 +212,28 @@ constexpr int SW_ACC = 4 * SW_COLS + 2;      // min X, max S, min S, max Z per c
 // ---- candidate i is the positions (cuts[i-1], cuts[i]]; pattern incidences of a
 // position: the edges (triangles) of its vertex.
 
+// *rows: 1 + the last position whose vertex has a pattern
 __global__ void sg_positions_kernel(const int64_t* R, const int32_t* order, int32_t n, const int64_t* ptr, int32_t nact,
-                                    int64_t* Rp, int64_t* icnt, unsigned long long* acc) {
+                                    int64_t* Rp, int64_t* icnt, unsigned long long* acc, int32_t* rows) {
     if (blockIdx.x == 0 && threadIdx.x < SW_ACC) {
         const int i = threadIdx.x, kind = i < 4 * SW_COLS ? i / SW_COLS : i - 4 * SW_COLS + 2;
         acc[i] = (kind & 1) ? 0ull : ~0ull;      // the first window's extremes
     }
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int32_t last = 0;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= n; p += stride) {
         if (p == n) {
             icnt[p] = 0;
             continue;
         }
         const int32_t x = order[p];
+        const int64_t c = (ptr && x < nact) ? ptr[x + 1] - ptr[x] : 0;
         Rp[p] = R[x];
-        icnt[p] = (ptr && x < nact) ? ptr[x + 1] - ptr[x] : 0;
+        icnt[p] = c;
+        if (c) last = (int32_t)p + 1;
     }
+    last = __reduce_max_sync(0xffffffffu, last);
+    if ((threadIdx.x & 31) == 0 && last > *rows) atomicMax(rows, last);
 }
 
 // A pattern's change of the loads for a segment S, from where each member lies
@@ -280,7 +286,11 @@ __device__ __forceinline__ void pattern_delta(const int (&side)[3], const int32_
 // keeps the extremes of X, S and Z for column j.  Rows that no pattern of the
 // window touched hold one load throughout, so the rows touched earlier in the
 // chain (list M) add one minimum (S) and one maximum (Z), and the unmodified rest
-// of Z is at most its first position's load.  Then every block takes the same
+// of Z is at most its first position's load.  Positions past the last one with a
+// pattern (isolated vertices, for triangles those in none) never change and have no
+// row: their extremes are the sorted loads at the ends of their range.  (With a row for
+// each, 50,000 vertices of 2^23 took a table of 268 MB, and windows of 4 because of it:
+// over 50 s after binary64 iterations, 2.2 s so.)  Then every block takes the same
 // decision from the 4 x 32 extremes: the first column that accepts or fails on
 // the X side ends the chain there, else the next window continues it.
 //
@@ -301,11 +311,12 @@ struct SgWalkArgs {
     const int32_t *vt_idx, *ta, *tb, *tc;
     const int64_t* W;
     int64_t Dn;
-    int32_t n, ncand, cols;
+    int32_t n, ncand, cols, maxrows;
+    const int32_t* rows;                      // 1 + the last position with a pattern
     int64_t cap0, max_windows;
-    long long* table;                         // [n][cols], zero between windows
-    int64_t* delta;                           // [n] change of a position's load, valid when dstamp is the chain's
-    int32_t *stamp, *dstamp;                  // [n] window (chain) that last touched the position
+    long long* table;                         // [maxrows][cols], zero between windows
+    int64_t* delta;                           // [maxrows] change of a position's load, valid when dstamp is the chain's
+    int32_t *stamp, *dstamp;                  // [maxrows] window (chain) that last touched the position
     int32_t *list, *mlist;                    // rows touched in this window; positions touched in this chain
     unsigned long long* acc;                  // [3][SW_ACC]
     int32_t* cnt;                             // [0..2] list counts, [3] mlist count
@@ -393,7 +404,11 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
     __shared__ unsigned long long s_rX, s_rS;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + tid, nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int32_t n = A.n;
+    const int32_t n = A.n, P = *A.rows;
+    if (P > A.maxrows) {                                 // (vertices with patterns have loads: they sort first)
+        if (gtid == 0) A.out[1] = 2;
+        return;
+    }
     if (tid == 0) {
         s_start = 0;
         s_b0 = -1;
@@ -444,7 +459,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
         const bool cmode = s_chainmode != 0;
         const SgTouch T{A, win + 1, A.cnt + win % 3};
         // phase 1
-        for (int64_t p = (int64_t)b0 + 1 + gtid; p <= bw; p += nthreads) T.mark((int32_t)p);
+        for (int64_t p = (int64_t)b0 + 1 + gtid; p <= min(bw, P - 1); p += nthreads) T.mark((int32_t)p);
         const int64_t i1 = A.ioff[bw + 1];
         for (int64_t i = A.ioff[b0 + 1] + gtid; i < i1; i += nthreads) {
             int32_t lo = b0 + 1, hi = bw + 1;            // the last position with ioff <= i
@@ -566,12 +581,17 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
             unsigned long long mx = __ldcg(acc + lane), hi = __ldcg(acc + SW_COLS + lane);
             unsigned long long lo = __ldcg(acc + 2 * SW_COLS + lane), mz = __ldcg(acc + 3 * SW_COLS + lane);
             const int32_t sa = cmode ? a : la;
+            if (act && lb >= P) {                        // S reaches past the rows
+                hi = max(hi, (unsigned long long)A.Rp[max(sa, P)]);
+                lo = min(lo, (unsigned long long)A.Rp[lb]);
+            }
             if (cmode) {
                 mx = min(mx, s_rX);
                 hi = max(hi, s_rS);
                 lo = min(lo, __ldcg(acc + 4 * SW_COLS));
                 mz = max(mz, __ldcg(acc + 4 * SW_COLS + 1));
-                if (bw + 1 < n) mz = max(mz, (unsigned long long)A.Rp[bw + 1]);
+                const int32_t q = max(lb + 1, min(bw + 1, P));          // first of Z that no row stands for
+                if (act && q < n) mz = max(mz, (unsigned long long)A.Rp[q]);
             } else if (act) {
                 if (la > 0) mx = min(mx, (unsigned long long)A.Rp[la - 1]);
                 if (lb + 1 < n) mz = max(mz, (unsigned long long)A.Rp[lb + 1]);
@@ -718,20 +738,23 @@ static void sg_walk(lds_graph* g, SgState& st, const int64_t* cand) {
     else ensure_edge_shift(g);
     const int64_t* ptr = tri ? (g->ntri > 0 ? g->vt_ptr.get() : nullptr) : (g->m > 0 ? g->rowptr.get() : nullptr);
     const int64_t incid = tri ? 3 * std::max<int64_t>(g->ntri, 0) : 2 * g->m;
-    // Table columns: 32 (256 B per position, against the 96 B per vertex and edge a
-    // query is admitted with), fewer past 2^20 positions so that the table stays
-    // within 256 MB; never under 4, so that a long chain still moves in windows.
-    int32_t cols = (int32_t)std::max<int64_t>(4, std::min<int64_t>(SW_COLS, ((int64_t)1 << 25) / n));
+    // Rows: vertices with a pattern have loads above zero, so they sort before the others.
+    // Table columns: 32, fewer where that is more than 64 B per vertex and edge (two thirds
+    // of the 96 a query is admitted with; fewer than 3 edges a vertex) or than 8 GB, never
+    // under 4, so that a long chain still moves in windows.
+    const int32_t rows = std::max(1, std::min(n, g->nact));
+    const int64_t bytes = std::min<int64_t>(64 * (g->m + n) + (1 << 20), (int64_t)1 << 33);
+    int32_t cols = (int32_t)std::max<int64_t>(4, std::min<int64_t>(SW_COLS, bytes / 8 / rows));
     if (g_sg_variant.load(std::memory_order_relaxed) == 1) cols = 1;
-    DevBuf<int64_t> Rp(n, s), icnt(n + 1, s), delta(n, s);
-    DevBuf<long long> table((size_t)n * cols, s);
-    DevBuf<int32_t> stamps(2 * (size_t)n, s), lists(2 * (size_t)n, s), ctl(8, s);
+    DevBuf<int64_t> Rp(n, s), icnt(n + 1, s), delta(rows, s);
+    DevBuf<long long> table((size_t)rows * cols, s);
+    DevBuf<int32_t> stamps(2 * (size_t)rows, s), lists(2 * (size_t)rows, s), ctl(9, s);
     DevBuf<unsigned long long> acc(3 * SW_ACC, s);
-    LDS_CUDA(cudaMemsetAsync(table.get(), 0, (size_t)n * cols * sizeof(long long), s));
-    LDS_CUDA(cudaMemsetAsync(stamps.get(), 0, 2 * (size_t)n * sizeof(int32_t), s));
-    LDS_CUDA(cudaMemsetAsync(ctl.get(), 0, 8 * sizeof(int32_t), s));
+    LDS_CUDA(cudaMemsetAsync(table.get(), 0, (size_t)rows * cols * sizeof(long long), s));
+    LDS_CUDA(cudaMemsetAsync(stamps.get(), 0, 2 * (size_t)rows * sizeof(int32_t), s));
+    LDS_CUDA(cudaMemsetAsync(ctl.get(), 0, 9 * sizeof(int32_t), s));
     LDS_LAUNCH(sg_positions_kernel, grid_for(n + 1, 256), 256, 0, s, g->fw_R.get(), st.order.get(), n, ptr, g->nact,
-               Rp.get(), icnt.get(), acc.get());
+               Rp.get(), icnt.get(), acc.get(), ctl.get() + 8);
     exclusive_scan_i64_dev(icnt.get(), icnt.get(), (int64_t)n + 1, nullptr, s);
     st.gend.alloc(ncut, s);
     st.lo.alloc(ncut, s);
@@ -760,14 +783,16 @@ static void sg_walk(lds_graph* g, SgState& st, const int64_t* cand) {
     A.n = n;
     A.ncand = (int32_t)ncut;
     A.cols = cols;
+    A.maxrows = rows;
+    A.rows = ctl.get() + 8;
     A.cap0 = 2 * (int64_t)grid * SW_THREADS;
     A.max_windows = 2 * ncut + 64;           // every second window at least decides a candidate
     A.table = table.get();
     A.delta = delta.get();
     A.stamp = stamps.get();
-    A.dstamp = stamps.get() + n;
+    A.dstamp = stamps.get() + rows;
     A.list = lists.get();
-    A.mlist = lists.get() + n;
+    A.mlist = lists.get() + rows;
     A.acc = acc.get();
     A.cnt = ctl.get();
     A.gend = st.gend.get();
@@ -780,6 +805,7 @@ static void sg_walk(lds_graph* g, SgState& st, const int64_t* cand) {
     int32_t h[4];
     LDS_CUDA(cudaMemcpyAsync(h, ctl.get() + 4, sizeof(h), cudaMemcpyDeviceToHost, s));
     LDS_CUDA(cudaStreamSynchronize(s));
+    LDS_REQUIRE(h[1] != 2, LDS_ECUDA, "extract_sg: a vertex with patterns has no load (internal error)");
     LDS_REQUIRE(h[1] == 0, LDS_ETIMEOUT, "extract_sg: the walk hit its window bound");
     st.ng = h[0];
     st.windows = h[2];
