@@ -290,7 +290,7 @@ __device__ __forceinline__ void pattern_delta(const int (&side)[3], const int32_
 // pattern (isolated vertices, for triangles those in none) never change and have no
 // row: their extremes are the sorted loads at the ends of their range.  (With a row for
 // each, 50,000 vertices of 2^23 took a table of 268 MB, and windows of 4 because of it:
-// over 50 s after binary64 iterations, 2.2 s so.)  Then every block takes the same
+// over 50 s after binary64 iterations, 1.6 s so.)  Then every block takes the same
 // decision from the 4 x 32 extremes: the first column that accepts or fails on
 // the X side ends the chain there, else the next window continues it.
 //
