@@ -92,8 +92,21 @@ int32_t lds_device_count(void);
 lds_status lds_create_graph(int32_t n, int64_t m, const int32_t* src, const int32_t* dst,
                             lds_mem where, void* stream, lds_graph** out);
 
-/* Releases every device buffer of the handle (NULL is ignored). */
+/* Releases every device buffer of the handle (NULL is ignored), after the work
+ * on its stream.  The library keeps released device memory for its next call, out
+ * of reach of other allocators in the process: at most 1/16 of the device's memory
+ * while a handle made on that device is alive, 1/32 once none is (see
+ * lds_release_memory). */
 void lds_free(lds_graph* g);
+
+/* Gives all device memory that the library holds and does not use back to the
+ * driver, on every device; waits for the devices' work.  Errors: LDS_ECUDA. */
+lds_status lds_release_memory(void);
+
+/* Bytes of device memory that the library holds on the current device, that its
+ * buffers use, and the most that they used since the last call that asked for
+ * `peak` (any may be NULL).  Errors: LDS_ECUDA. */
+lds_status lds_memory_info(int64_t* held, int64_t* in_use, int64_t* peak);
 
 lds_status lds_graph_info(const lds_graph* g, lds_graph_info_t* info);
 

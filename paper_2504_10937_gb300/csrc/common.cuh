@@ -81,9 +81,10 @@ extern int g_fail_alloc_countdown;
 
 void* dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void* p, cudaStream_t s);
-// A graph handle begins or ends (the memory kept for the next call shrinks with the last one).
-void handle_created();
-void handle_freed();
+// A graph handle begins on the current device, which is returned, or ends (the memory
+// kept for the next call shrinks with the device's last one).
+int handle_created();
+void handle_freed(int device);
 
 // RAII device buffer allocated stream-ordered.
 template <class T>

@@ -363,12 +363,12 @@ lds_status lds_create_graph(int32_t n, int64_t m, const int32_t* src, const int3
         LDS_REQUIRE(lds_device_count() > 0, LDS_ECUDA, "lds_create_graph: no CUDA device");
         lds_graph* g = new lds_graph();
         g->stream = (cudaStream_t)stream;
-        handle_created();
+        const int dev = g->device = handle_created();
         try {
             build_graph(g, n, m, src, dst, where);
         } catch (...) {
             delete g;
-            handle_freed();
+            handle_freed(dev);
             throw;
         }
         *out = g;
@@ -377,10 +377,12 @@ lds_status lds_create_graph(int32_t n, int64_t m, const int32_t* src, const int3
 
 void lds_free(lds_graph* g) {
     if (!g) return;
-    cudaStreamSynchronize(g->stream);
+    const cudaStream_t s = g->stream;
+    const int dev = g->device;
+    cudaStreamSynchronize(s);
     delete g;
-    cudaStreamSynchronize(nullptr);
-    handle_freed();
+    cudaStreamSynchronize(s);          // its buffers are free now, and can be given back
+    handle_freed(dev);
 }
 
 lds_status lds_graph_info(const lds_graph* g, lds_graph_info_t* info) {

@@ -14,6 +14,7 @@ struct lds_graph {
     int32_t nact = 0;     // non-isolated vertices (internal ids 0..nact-1)
     int64_t m = 0;        // distinct undirected edges
     cudaStream_t stream = nullptr;
+    int device = -1;      // the device it was made on
     lds_graph_info_t info{};
 
     lds::DevBuf<int32_t> to_orig;     // [n] internal -> original

@@ -106,6 +106,8 @@ def load():
                                                    ctypes.POINTER(i64), ctypes.POINTER(ctypes.c_char_p)])
     _sig(lib, "lds_set_pass_profiling", None, [i32])
     _sig(lib, "lds_debug_fail_alloc_after", None, [i32])
+    _sig(lib, "lds_release_memory", ctypes.c_int, [])
+    _sig(lib, "lds_memory_info", ctypes.c_int, [ctypes.POINTER(i64), ctypes.POINTER(i64), ctypes.POINTER(i64)])
     _sig(lib, "lds_launch_count", i64, [])
     _sig(lib, "lds_set_fw_variant", ctypes.c_int, [i32])
     _sig(lib, "lds_set_flow_variant", ctypes.c_int, [i32])
@@ -179,6 +181,19 @@ def set_flow_variant(variant: int):
 def set_extract_variant(variant: int):
     """0: windows of up to 32 candidates; 1: windows of one candidate."""
     _check(load().lds_set_extract_variant(int(variant)))
+
+
+def release_memory():
+    """Gives the device memory that the library keeps unused back to the driver."""
+    _check(load().lds_release_memory())
+
+
+def memory_info() -> dict:
+    """Device memory of the library on the current device: held from the driver, in use,
+    and the most in use since the last call (bytes)."""
+    h, u, p = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_int64()
+    _check(load().lds_memory_info(ctypes.byref(h), ctypes.byref(u), ctypes.byref(p)))
+    return {"held": h.value, "in_use": u.value, "peak": p.value}
 
 
 def launch_count() -> int:
