@@ -741,7 +741,9 @@ static void sg_walk(lds_graph* g, SgState& st, const int64_t* cand) {
     // Rows: vertices with a pattern have loads above zero, so they sort before the others.
     // Table columns: 32, fewer where that is more than 64 B per vertex and edge (two thirds
     // of the 96 a query is admitted with; fewer than 3 edges a vertex) or than 8 GB, never
-    // under 4, so that a long chain still moves in windows.
+    // under 4, so that a long chain still moves in windows.  The other arrays take 64 B per
+    // vertex and 32 per row.  Keeping the sum within the 96 would leave 15 columns at 2^20
+    // vertices with 200k edges, 300 ms against 164 with 30 (249 with a row for every vertex).
     const int32_t rows = std::max(1, std::min(n, g->nact));
     const int64_t bytes = std::min<int64_t>(64 * (g->m + n) + (1 << 20), (int64_t)1 << 33);
     int32_t cols = (int32_t)std::max<int64_t>(4, std::min<int64_t>(SW_COLS, bytes / 8 / rows));
@@ -871,6 +873,9 @@ void extract_sg(lds_graph* g, SgState& st) {
     st.ncut = exclusive_scan_i32_to_i64(flag.get(), fex.get(), n, s);
     st.cuts.alloc(std::max<int64_t>(st.ncut, 1), s);
     LDS_LAUNCH(cut_list_kernel, grid_for(n, blk), blk, 0, s, flag.get(), fex.get(), n, st.cuts.get());
+    h.release();
+    incl.release();
+    flag.release();
     // 4. the candidate walk (the last position is always a cut, so ncut >= 1)
     const double ms_cuts = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
     sg_walk(g, st, fex.get());

@@ -1,5 +1,6 @@
 """Device memory that the library keeps between calls: how much is held and used, that it
-is given back, and that a reset device starts anew."""
+is given back, that a reset device starts anew, and that the walk of ExtractSG keeps to
+its bound."""
 import os
 import subprocess
 import sys
@@ -92,3 +93,17 @@ def test_a_reset_device_starts_anew():
     env["LD_LIBRARY_PATH"] = "/usr/local/cuda/lib64:" + env.get("LD_LIBRARY_PATH", "")
     out = subprocess.run([sys.executable, "-c", RESET], env=env, cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert out.returncode == 0 and "reset ok" in out.stdout, out.stdout + out.stderr
+
+
+@pytest.mark.parametrize("n,m", [(1 << 20, 200_000), (1 << 22, 100_000), (300_000, 150_000)])
+def test_the_walk_keeps_to_its_bound(lds, n, m):
+    # the table 64 B per edge and vertex and 1 MB, its other arrays 64 B per vertex and 32 per
+    # active one, 8 more for the edges' numbers that stay on the handle; 256 B more a buffer
+    with lds.Graph(*_random(n, m, 4)) as g:
+        g.fw(30, want=())
+        nact = n - g.info()["isolated"]
+        before = lds.memory_info()["in_use"]
+        lds.memory_info()
+        g.extract_sg()
+        grown = lds.memory_info()["peak"] - before
+        assert grown <= 64 * (g.m + n) + (1 << 20) + 64 * n + 40 * nact + 32 * 256

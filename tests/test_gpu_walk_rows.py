@@ -1,6 +1,6 @@
 """The ExtractSG walk where positions have no row of their own (isolated vertices,
-vertices in no triangle) and where its table has between 4 and 32 columns (fewer than
-three edges a vertex): against the oracle and against windows of one candidate."""
+vertices in no triangle) and where its table has between 4 and 32 columns (few edges
+a vertex): against the oracle and against windows of one candidate."""
 import time
 from fractions import Fraction
 
