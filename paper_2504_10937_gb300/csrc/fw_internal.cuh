@@ -46,12 +46,20 @@ struct PassTimer {
 };
 
 // Number of iterations whose bit planes are kept before folding: at most
-// ~2 GiB of planes, between 32 and 512 iterations, never more than N.
-inline int planes_capacity(int64_t plane_words, int N) {
-    int64_t budget = (int64_t)2 << 30;
+// ~2 GiB of planes and `most` bytes, between 32 and 512 iterations, never more than N.
+inline int planes_capacity(int64_t plane_words, int N, int64_t most = (int64_t)2 << 30) {
+    const int64_t budget = std::min((int64_t)2 << 30, most);
     int64_t cap = plane_words > 0 ? budget / (plane_words * 4) : N;
     cap = std::max<int64_t>(32, std::min<int64_t>(cap, 512));
     return (int)std::min<int64_t>(cap, std::max(N, 1));
+}
+
+// Bytes of planes for `items` choices of `bits` bits in quads: half as much again as 512
+// iterations of whole quads take, so that rows and groups of few entries, up to four
+// times the quads, do not take four times the memory (a perfect matching of 2^20
+// vertices: 134 MB of planes, where a bit per choice is 34).
+inline int64_t quad_plane_bytes(int64_t items, int bits) {
+    return std::max<int64_t>((int64_t)16 << 20, 96 * items * bits);
 }
 
 // Folds `nplanes` bit planes (plane k at planes + k * nchunks, bit l of word g

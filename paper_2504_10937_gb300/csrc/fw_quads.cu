@@ -433,7 +433,7 @@ bool run_edge_fw_quads(lds_graph* g, int N, lds_precision p, bool want_last, Pas
     LDS_CUDA(cudaMemsetAsync(cnt.get(), 0, ((size_t)nact + 1) * sizeof(uint32_t), s));
     LDS_LAUNCH(eq_init_kernel, grid_for(nact + 1, blk), blk, 0, s, g->rowptr.get(), g->fwv_perm.get(), nact, w32.get(),
                r32.get(), R.get());
-    const int K = planes_capacity(4 * nchunks, N);
+    const int K = planes_capacity(4 * nchunks, N, quad_plane_bytes(m, 1));
     DevBuf<uint4> planes(std::max<int64_t>(1, (int64_t)K * nchunks), s);
     DevBuf<uint32_t> W(128 * nchunks, s);
     LDS_CUDA(cudaMemsetAsync(W.get(), 0, 128 * nchunks * sizeof(uint32_t), s));

@@ -416,7 +416,7 @@ void run_tri_fw(lds_graph* g, int N, lds_precision p, bool want_last, PassTimer&
     DevBuf<uint32_t> cnt((size_t)nact + 1, s);
     LDS_CUDA(cudaMemsetAsync(cnt.get(), 0, ((size_t)nact + 1) * sizeof(uint32_t), s));
     LDS_LAUNCH(tq_init_kernel, grid_for(nact, blk), blk, 0, s, g->tv_count.get(), nact, r32.get(), R.get());
-    const int K = planes_capacity(8 * nchunks, N);
+    const int K = planes_capacity(8 * nchunks, N, quad_plane_bytes(nt, 2));
     DevBuf<uint4> planes(std::max<int64_t>(1, 2 * (int64_t)K * nchunks), s);
     DevBuf<uint32_t> Wb(items, s), Wc(items, s);
     LDS_CUDA(cudaMemsetAsync(Wb.get(), 0, items * sizeof(uint32_t), s));

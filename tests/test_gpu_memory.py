@@ -1,6 +1,6 @@
 """Device memory that the library keeps between calls: how much is held and used, that it
-is given back, that a reset device starts anew, and that the walk of ExtractSG keeps to
-its bound."""
+is given back, that a reset device starts anew, and that the walk of ExtractSG and the
+choice planes of Frank-Wolfe keep to their bounds."""
 import os
 import subprocess
 import sys
@@ -107,3 +107,25 @@ def test_the_walk_keeps_to_its_bound(lds, n, m):
         g.extract_sg()
         grown = lds.memory_info()["peak"] - before
         assert grown <= 64 * (g.m + n) + (1 << 20) + 64 * n + 40 * nact + 32 * 256
+
+
+def test_planes_of_padded_quads_keep_to_their_bound(lds):
+    # one target a row, one triangle a group: every quad holds one entry.  Planes, weights
+    # per entry (16 B a quad and plane set), loads and counts of the vertices, and the
+    # results themselves, of which the last are replaced
+    n = 1 << 20
+    with lds.Graph(n, np.arange(0, n, 2, dtype=np.int32), np.arange(1, n, 2, dtype=np.int32)) as g:
+        g.fw(1, want=())
+        before = lds.memory_info()["in_use"]
+        lds.memory_info()
+        g.fw(600, want=())
+        assert g.fw_timing()["pass_kernel"] == "fw_quad_kernel"
+        assert lds.memory_info()["peak"] - before <= (96 + 16) * g.m + 16 * n + (1 << 20)
+    t = 300_000
+    b = np.arange(0, 3 * t, 3, dtype=np.int32)
+    with lds.Graph(3 * t, np.r_[b, b, b + 1], np.r_[b + 1, b + 2, b + 2]) as g:
+        g.fw(1, density="triangle", want=())
+        before = lds.memory_info()["in_use"]
+        lds.memory_info()
+        g.fw(600, density="triangle", want=())
+        assert lds.memory_info()["peak"] - before <= (192 + 32) * t + 16 * 3 * t + (1 << 20)
