@@ -487,10 +487,8 @@ void fw_run(lds_graph* g, lds_density d, int32_t iters, lds_precision p, bool wa
         bool res = false;
         if (g_fw_variant == 0 || g_fw_variant == 6) {
             if (want_last) g->fw_last.alloc(std::max<int64_t>(g->m, 1), s);
-            timer.start(s);
-            res = fw_resident_run(g, iters, p, want_last ? g->fw_last.get() : nullptr);
-            if (res) timer.stop(s, iters);
-            else g->fw_last.release();
+            res = fw_resident_run(g, iters, p, want_last ? g->fw_last.get() : nullptr, timer);
+            if (!res) g->fw_last.release();
         }
         const bool quads = !res && (g_fw_variant == 0 || g_fw_variant == 5 || g_fw_variant == 6) &&
                            run_edge_fw_quads(g, iters, p, want_last, timer);

@@ -28,7 +28,7 @@
 
 #include <algorithm>
 
-#include "graph.cuh"
+#include "fw_internal.cuh"
 
 namespace lds {
 
@@ -349,7 +349,7 @@ const void* res64_kernel(int U) {
 }
 
 // launch of either form over G CTAs
-void res_launch(const void* fn, int G, ResSync sync, size_t smem, void** args, cudaStream_t s) {
+void res_launch(const void* fn, int G, ResSync sync, size_t smem, void** args, int N, PassTimer& timer, cudaStream_t s) {
     LDS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RES_SMEM));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(G);
@@ -367,14 +367,16 @@ void res_launch(const void* fn, int G, ResSync sync, size_t smem, void** args, c
     }
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    timer.start(s);
     LDS_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
     g_launches.fetch_add(1, std::memory_order_relaxed);
+    timer.stop(s, N);
 }
 
 }  // namespace
 
 // The binary64 form; false when the graph does not fit.
-static bool fw_resident64_run(lds_graph* g, int32_t N, uint8_t* last) {
+static bool fw_resident64_run(lds_graph* g, int32_t N, uint8_t* last, PassTimer& timer) {
     const int64_t maxdeg = std::max(g->info.max_degree, 1), slots = 2 * g->m;
     // CTAs: one up to 1,024 slots, a cluster of 8 up to 8,192, then one per 1,024 slots
     constexpr int64_t kShare = 1024;
@@ -399,13 +401,13 @@ static bool fw_resident64_run(lds_graph* g, int32_t N, uint8_t* last) {
     Res64Args A{g->rowptr.get(), g->col.get(),  g->edge_shift.get(), g->nact, N, words.get(),
                 g->fw_W.get(),   g->fw_R.get(), g->fw_r.get(),       last};
     void* args[] = {(void*)&A};
-    res_launch(fn, G, sync, smem, args, s);
+    res_launch(fn, G, sync, smem, args, N, timer, s);
     return true;
 }
 
-bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last) {
+bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last, PassTimer& timer) {
     if (N < 1 || g->m < 1 || g->nact > 65536) return false;
-    if (p == LDS_FP64) return fw_resident64_run(g, N, last);
+    if (p == LDS_FP64) return fw_resident64_run(g, N, last, timer);
     const bool fp32 = p == LDS_FP32;
     const int64_t maxdeg = std::max(g->info.max_degree, 1), slots = 2 * g->m;
     const unsigned __int128 D = (unsigned __int128)(N + 1) * (unsigned __int128)(N + 2);
@@ -444,7 +446,7 @@ bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last) {
     ResArgs A{g->rowptr.get(), g->col.get(),   g->edge_shift.get(), g->nact, N, words.get(),
               g->fw_W.get(),   g->fw_R.get(),  g->fw_r.get(),       last};
     void* args[] = {(void*)&A};
-    res_launch(fn, G, sync, smem, args, s);
+    res_launch(fn, G, sync, smem, args, N, timer, s);
     return true;
 }
 

@@ -134,11 +134,12 @@ void to_original_order_f64(const lds_graph* g, const double* in_int, double* out
 // Batched on-chip Frank-Wolfe (fw_batch.cu): tunes the threads per graph of every
 // size bucket among the given graphs (kept for the process), and reports the choice.
 void fw_batch_autotune(int32_t count, lds_graph** graphs, int32_t iters, lds_precision p);
+struct PassTimer;
 // lds_fw's edge-density iterations of a graph whose slots fit the chip's registers
 // (fw_resident.cu); fills the handle's R, r, W and, when `last` is given, the last
 // iteration's choices.  False when the graph does not fit (the caller runs another
 // path).
-bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last);
+bool fw_resident_run(lds_graph* g, int32_t N, lds_precision p, uint8_t* last, PassTimer& timer);
 int32_t fw_batch_threads(int32_t nact);
 
 }  // namespace lds
