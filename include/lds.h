@@ -353,7 +353,9 @@ typedef struct {
 /* Starts `workers` worker threads on the current device with a device-memory
  * budget of `budget_bytes` for the queries in flight.  A query's footprint is
  * estimated as 96 B per edge and per vertex plus 64 B per triangle for LTDS
- * (16 per edge stands in for |T| while the triangles are not listed yet).
+ * (16 per edge stands in for |T| while the triangles are not listed yet): a
+ * rough figure, the peak of a query beside its handle is 0.4 to 2 times that
+ * (lds_memory_info), so a budget is best kept at half of the free memory.
  * Errors: LDS_EINVAL, LDS_ECUDA. */
 lds_status lds_server_create(int64_t budget_bytes, int32_t workers, lds_server** out);
 
@@ -399,7 +401,8 @@ int32_t lds_debug_pick_next(int32_t nq, const int64_t* bytes, const uint8_t* gra
  * otherwise and under any other variant but 6):
  *   0  automatic: a graph of at most 65,536 active vertices whose symmetric
  *      CSR slots fit the chip's registers (up to 16,384 per CTA, rows whole;
- *      the load words in shared memory, at most 57,344 vertices; every weight
+ *      the load words of all vertices and the receipt counts of a CTA's rows in
+ *      224 KB of shared memory, so some 50,000 to 57,000 vertices; every weight
  *      and exact load below 2^32) runs with its slots resident, each endpoint
  *      deciding its own edges, one barrier per iteration over one CTA, a
  *      cluster of 8 or up to one CTA per SM; otherwise the degree-oriented
@@ -437,7 +440,8 @@ lds_status lds_set_flow_variant(int32_t variant);
 /* ExtractSG walk (Alg. 2's merge loop) for lds_extract_sg and lds_topk
  * (process-wide).  The walk runs on the device in one cooperative launch that
  * decides a window of candidates at a time:
- *   0  automatic: windows of up to 32 candidates;
+ *   0  automatic: windows of up to 32 candidates (fewer, at least 4, where a
+ *      table of 32 columns would take more than 64 B per vertex and edge);
  *   1  windows of one candidate.
  * Both give the same groups and bounds.  Errors: LDS_EINVAL. */
 lds_status lds_set_extract_variant(int32_t variant);

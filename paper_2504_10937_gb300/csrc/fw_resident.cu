@@ -23,7 +23,9 @@
 // the grid-wide pass (GB300): 1,500 vertices with 348k edges 10.4 -> 3.2 us, 40,000
 // with 240k edges 10.3 -> 4.2 us, 6,000 with 24k edges 8.1 -> 2.4 us, 300 with 1,500
 // edges 4.9 -> 0.85 us (the 8-CTA form that counted both endpoints in shared memory
-// took 2.6 us at 2k edges and 5 at 32k).
+// took 2.6 us at 2k edges and 5 at 32k).  With 16 slots a thread the registers spill
+// (96 to 128 B); 2M slots on 20,000 vertices still take 7.4 us against 9.0 by the pass
+// over quads, 1.6M on 8,000 5.6 against 9.0.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -378,7 +380,10 @@ void res_launch(const void* fn, int G, ResSync sync, size_t smem, void** args, i
 // The binary64 form; false when the graph does not fit.
 static bool fw_resident64_run(lds_graph* g, int32_t N, uint8_t* last, PassTimer& timer) {
     const int64_t maxdeg = std::max(g->info.max_degree, 1), slots = 2 * g->m;
-    // CTAs: one up to 1,024 slots, a cluster of 8 up to 8,192, then one per 1,024 slots
+    // CTAs: one up to 1,024 slots, a cluster of 8 up to 8,192, then one per 1,024 slots, by
+    // microseconds an iteration (300 iterations, GB300) of one CTA, a cluster and the grid:
+    // 480 slots 3.5, 3.1; 1,800 9.2, 4.5, 7.9; 7,300 14.4, 8.5, 9.2; 10,000 15.5, 11.1, 11.2;
+    // 16,700 16.5, 15.0, 12.2; 29,000 20.6, 21.8, 14.0
     constexpr int64_t kShare = 1024;
     int G = slots <= kShare ? 1
             : slots <= RES_CLUSTER * kShare ? RES_CLUSTER : (int)std::min<int64_t>(num_sms(), (slots + kShare - 1) / kShare);

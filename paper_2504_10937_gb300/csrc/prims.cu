@@ -390,11 +390,6 @@ __global__ void __launch_bounds__(RS_SMALL_T, 1) rs_small_kernel(Key* keys, uint
     }
 }
 
-__global__ void gather_u32_kernel(const uint32_t* in, const uint32_t* idx, uint32_t* out, int64_t n) {
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = in[idx[i]];
-}
-
 }  // namespace
 
 template <class Key, bool VALS>
@@ -444,12 +439,6 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaStr
 
 void radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s) {
     radix_sort<uint32_t, true>(keys, vals, n, bits, s);
-}
-
-void gather_u32(const uint32_t* in, const uint32_t* idx, uint32_t* out, int64_t n, cudaStream_t s) {
-    if (n <= 0) return;
-    LDS_LAUNCH(gather_u32_kernel, grid_for(n, 256), 256, 0, s, in, idx, out, n);
-    LDS_CHECK_LAUNCH();
 }
 
 }  // namespace lds

@@ -26,7 +26,4 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, cudaStr
 // 32-bit keys; vals must be given.
 void radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int bits, cudaStream_t s);
 
-// Gathers: out[i] = in[idx[i]].
-void gather_u32(const uint32_t* in, const uint32_t* idx, uint32_t* out, int64_t n, cudaStream_t s);
-
 }  // namespace lds

@@ -5,8 +5,9 @@
 // to the higher one, which bounds out-degrees by O(sqrt(m)); each oriented edge
 // x -> y meets out(x) and out(y) (both ascending) by a merge walk, and each
 // common out-neighbour w closes the triangle {x, y, w} exactly once.  A count
-// pass sizes the output, a write pass fills it, and two stable radix sorts put
-// the rows in (a, b, c) order.
+// pass sizes the output, a write pass fills it, and a radix sort puts the rows in
+// (a, b, c) order: one of the packed triangles up to 2^21 vertices, two stable ones
+// with payload past them.
 //
 // Core numbers: level-synchronous peeling.  At level k every live vertex whose
 // remaining degree (number of live triangles for tr-core) is <= k gets core k
