@@ -38,7 +38,9 @@ std::atomic<long long> g_launches{0};
 // as they shared the default pool.
 //
 // A pool dies with its context (cudaDeviceReset), so it is known by the context's id,
-// which is never used again, and a context that has none yet gets one of its own.
+// which is never used again, and a context that has none yet gets one of its own.  The
+// look-up is made once per entry point and thread, at its first allocation (at every
+// allocation it cost about 1 % of a query of 6 ms).
 namespace {
 constexpr int kMaxDevices = 64;
 constexpr int kMaxContexts = 16;         // per device, over the process's life; then the default pool serves
@@ -168,6 +170,11 @@ void handle_freed(int dev) {
     });
 }
 
+static thread_local bool t_pool_known = false;
+static thread_local DevPool* t_pool = nullptr;
+
+void pool_forget() { t_pool_known = false; }
+
 void* dev_alloc(size_t bytes, cudaStream_t s) {
     if (g_fail_alloc_countdown > 0) {
         if (--g_fail_alloc_countdown == 0) {
@@ -176,7 +183,11 @@ void* dev_alloc(size_t bytes, cudaStream_t s) {
         }
     }
     void* p = nullptr;
-    DevPool* d = dev_pool(true);
+    if (!t_pool_known) {
+        t_pool = dev_pool(true);
+        t_pool_known = true;
+    }
+    DevPool* d = t_pool;
     cudaError_t e = d ? cudaMallocFromPoolAsync(&p, bytes, d->pool, s) : cudaMallocAsync(&p, bytes, s);
     if (e == cudaErrorMemoryAllocation && d) {
         cudaGetLastError();

@@ -56,9 +56,13 @@ extern std::atomic<long long> g_launches;
         }                                                                           \
     } while (0)
 
+// An entry point begins on this thread: the memory pool is looked up anew (common.cu).
+void pool_forget();
+
 // Wraps an entry point body: returns LDS_OK or the status of the first failure.
 template <class F>
 lds_status guard(F&& f) {
+    pool_forget();
     try {
         f();
         return LDS_OK;
