@@ -458,7 +458,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
         const bool cmode = s_chainmode != 0;
         const SgTouch T{A, win + 1, A.cnt + win % 3};
         // phase 1
-        for (int64_t p = (int64_t)b0 + 1 + gtid; p <= min(bw, P - 1); p += nthreads) T.mark((int32_t)p);
+        const int32_t bm = min(bw, P - 1);
+        for (int64_t p = (int64_t)b0 + 1 + gtid; p <= bm; p += nthreads) T.mark((int32_t)p);
         const int64_t i1 = A.ioff[bw + 1];
         for (int64_t i = A.ioff[b0 + 1] + gtid; i < i1; i += nthreads) {
             int32_t lo = b0 + 1, hi = bw + 1;            // the last position with ioff <= i
@@ -580,7 +581,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
             unsigned long long mx = __ldcg(acc + lane), hi = __ldcg(acc + SW_COLS + lane);
             unsigned long long lo = __ldcg(acc + 2 * SW_COLS + lane), mz = __ldcg(acc + 3 * SW_COLS + lane);
             const int32_t sa = cmode ? a : la;
-            if (act && lb >= P) {                        // S reaches past the rows
+            const bool past = bw >= P;                   // the window reaches past the rows
+            if (past && act && lb >= P) {
                 hi = max(hi, (unsigned long long)A.Rp[max(sa, P)]);
                 lo = min(lo, (unsigned long long)A.Rp[lb]);
             }
@@ -589,8 +591,9 @@ __global__ void __launch_bounds__(SW_THREADS, 1) sg_walk_kernel(const SgWalkArgs
                 hi = max(hi, s_rS);
                 lo = min(lo, __ldcg(acc + 4 * SW_COLS));
                 mz = max(mz, __ldcg(acc + 4 * SW_COLS + 1));
-                const int32_t q = max(lb + 1, min(bw + 1, P));          // first of Z that no row stands for
-                if (act && q < n) mz = max(mz, (unsigned long long)A.Rp[q]);
+                // the first position of Z that no row stands for
+                const int32_t q = past ? max(lb + 1, P) : bw + 1;
+                if (q < n) mz = max(mz, (unsigned long long)A.Rp[q]);
             } else if (act) {
                 if (la > 0) mx = min(mx, (unsigned long long)A.Rp[la - 1]);
                 if (lb + 1 < n) mz = max(mz, (unsigned long long)A.Rp[lb + 1]);
