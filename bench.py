@@ -47,7 +47,7 @@ UNIT_TRI = "triangle-updates/s"
 # from at capture time.  A kernel whose source changed since has no matching entry
 # and reports null.
 PASS_TRAFFIC = {
-    ("fw_quad_kernel", "exact", "0e232abe0d6ac3e0"): 4745357,     # profiles/fw_quad_chung_lu_1m.md
+    ("fw_quad_kernel", "exact", "262762dfa29b8fdf"): 4732045,     # profiles/fw_quad_chung_lu_1m.md
 }
 PASS_SOURCE = {"fw_opass32_kernel": "paper_2504_10937_gb300/csrc/fw_oriented.cu",
                "fw_quad_kernel": "paper_2504_10937_gb300/csrc/fw_quads.cu",
